@@ -40,27 +40,36 @@ struct Dims {
   static constexpr int NG = COLLOC ? NFP : (REDUCED ? N + 1 : (3 * N + 2) / 2);
 };
 
-// Operator block (element type T), packed by the host, staged in shared memory.
-// The per-element (surface, limiter) operators come first so a kernel that does
-// its volume contractions elsewhere can stage only [0, TAIL).
+// Operator block (element type T), packed by the host, staged in shared memory. The
+// per-element (face interpolation, limiter) operators come first so the limiter and
+// tensor-core kernels stage only [0, TAIL); the SIMT stage kernel stages a prefix (up to
+// DR with exact rules, up to PRT with the others, which need the nodal derivatives) and
+// its projection block (FP32 the rows PRT, PST, PT, FP64 PROJ4).
 template <int N>
 struct OpLayout {
   using D = Dims<N>;
-  static constexpr int LGT = 0;                                // [3 NG][NPP], Lg^T
-  static constexpr int I1D = LGT + 3 * D::NG * D::NPP;         // [NG][NFPP]
-  static constexpr int MW = I1D + D::NG * D::NFPP;             // [NPP] mean weights
+  static constexpr int QP = (3 * D::NG + 3) / 4 * 4;           // face points padded to fours
+  static constexpr int G4 = D::N == 2 ? (D::NCUB + 7) / 8 * 2 : (D::NCUB + 3) / 4;   // groups of 4 cubature points
+  static constexpr int I1D = 0;                                // [NG][NFPP]
+  static constexpr int I1P = I1D + D::NG * D::NFPP;            // [NG][NFPP][2] I1D rows of points g and NG-1-g
+  static constexpr int MW = I1P + 2 * D::NG * D::NFPP;         // [NPP] mean weights
   static constexpr int T1 = MW + D::NPP;                       // [3][NPP] P1 vertex map
   static constexpr int BARY = T1 + 3 * D::NPP;                 // [NPP][4] barycentric
   static constexpr int TAIL = BARY + 4 * D::NPP;
   static constexpr int IC = TAIL;                              // [NCUB][NPP]
   static constexpr int ICR = IC + D::NCUB * D::NPP;            // [NCUB][NPP]
   static constexpr int ICS = ICR + D::NCUB * D::NPP;           // [NCUB][NPP]
-  static constexpr int PRT = ICS + D::NCUB * D::NPP;           // [NCUB][NPP], Pr^T
+  static constexpr int WR = ICS + D::NCUB * D::NPP;            // [NPP][NPP] Pr Ic = M^-1 Dr^T M
+  static constexpr int WS = WR + D::NPP * D::NPP;              // [NPP][NPP] Ps Ic
+  static constexpr int LIFT4 = WS + D::NPP * D::NPP;           // [QP/4][NPP][4 points], -Lg
+  static constexpr int DR = LIFT4 + QP * D::NPP;               // [NPP][NPP] nodal d/dr
+  static constexpr int DS = DR + D::NPP * D::NPP;              // [NPP][NPP] nodal d/ds
+  static constexpr int PRT = DS + D::NPP * D::NPP;             // [NCUB][NPP], Pr^T
   static constexpr int PST = PRT + D::NCUB * D::NPP;           // [NCUB][NPP], Ps^T
   static constexpr int PT = PST + D::NCUB * D::NPP;            // [NCUB][NPP], P^T
-  static constexpr int DR = PT + D::NCUB * D::NPP;             // [NP][NPP] nodal d/dr
-  static constexpr int DS = DR + D::NP * D::NPP;               // [NP][NPP] nodal d/ds
-  static constexpr int SIZE = DS + D::NP * D::NPP;
+  static constexpr int PROJ4 = PT + D::NCUB * D::NPP;          // [G4][3 ops Pr,Ps,P][NPP][4 points]
+  static constexpr int LGT = PROJ4 + G4 * 3 * D::NPP * 4;      // [3 NG][NPP], Lg^T
+  static constexpr int SIZE = LGT + 3 * D::NG * D::NPP;
 };
 
 // Tensor-core tiling of the volume contractions (mma.sync, bf16 operands).
@@ -182,7 +191,7 @@ struct LimitParams : ScnParams<T> {
 
 constexpr int kBatchTile = 128;       // threads per CTA of the SIMT body (four warps, each taking its own
                                       // tickets); the tensor-core body runs the solvers' warps per CTA
-constexpr int kBatchStageTile = 64;   // elements per stage ticket: two warp-tiles
+constexpr int kBatchStageTile = 64;   // elements per stage ticket: whole warp-tiles of either body
 constexpr int kBatchTvbTile = 128;    // elements per TVB ticket: four per lane
 constexpr int kBatchMaxScn = 48;    // scenarios per group launch (kernel-parameter space)
 

@@ -1,13 +1,14 @@
 // Device kernels of the DG shallow-water right-hand side, the multirate
 // Adams-Bashforth update and the limiters (CUDA, sm_103a).
 //
-// One thread owns one element (element-blocked SIMT): the element's nodal state
-// stays in registers from the loads to the committed, limited result, and the
-// reference operators are staged once per CTA in shared memory, where every warp
-// reads them as broadcasts. Nodal arrays are node-major planes (node i of element
-// e at plane[i * KS + e]), so a warp's loads and stores of one node cover
-// consecutive elements: whole lines, and nearly so for the neighbour traces of
-// a mesh numbered with locality.
+// This file holds what the stage kernels share (traces, fluxes, Adams-Bashforth weights),
+// the limiter kernels and the pieces of the kernel-split ablation, where one thread owns
+// one element: its nodal state stays in registers, and the reference operators are
+// staged once per CTA in shared memory. The stage kernels themselves are in
+// kernels_team.cuh (SIMT, a team of lanes per element) and kernels_tc.cuh (tensor
+// cores). Nodal arrays are node-major planes (node i of element e at plane[i * KS + e]),
+// so a warp's loads and stores of one node cover consecutive elements: whole sectors,
+// and nearly so for the neighbour traces of a mesh numbered with locality.
 //
 // Formulation. The state is stored as (eta, hu, hv) with the free surface
 // eta = h + B. The momentum fluxes and the source are written about the datum
@@ -491,27 +492,6 @@ __device__ __forceinline__ void surface_fluxes(const StageParams<T>& p, const T*
   }
 }
 
-// Surface term with the lift R -= L^g F (Section 7.2) applied in registers, point
-// by point (the SIMT stage kernel).
-template <typename T, int N, bool kRolled = false, typename Own>
-__device__ __forceinline__ void surface_lift(const StageParams<T>& p, const T* __restrict__ sops, int e,
-                                             long long k, const Own& own, T rx, T ry, T sx, T sy, T md,
-                                             T (&R0)[Dims<N>::NP], T (&R1)[Dims<N>::NP],
-                                             T (&R2)[Dims<N>::NP]) {
-  using D = Dims<N>;
-  constexpr int NP = D::NP, NPP = D::NPP, NG = D::NG;
-  surface_fluxes<T, N, kRolled>(p, sops, e, k, own, rx, ry, sx, sy, md, [&](int f, int gq, T f0, T f1, T f2, T, T) {
-    T lg[NPP];
-    load_row<T, NPP>(sops + OpLayout<N>::LGT + (f * NG + gq) * NPP, lg);
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      R0[i] -= lg[i] * f0;
-      R1[i] -= lg[i] * f1;
-      R2[i] -= lg[i] * f2;
-    }
-  });
-}
-
 // The reference part of the pressure and source in strong form (element
 // reference split above): R_hu -= g h0 (r_x Dr + s_x Ds)(eta - eta0),
 // R_hv -= g h0 (r_y Dr + s_y Ds)(eta - eta0), h0 = eta0 - B0 the depth at node 0.
@@ -744,83 +724,6 @@ __device__ __forceinline__ void volume_term(const T* __restrict__ sops, const T 
       R2[i] += prt[i] * a2 + pst[i] * b2 + pt[i] * S2;
     }
   }
-}
-
-// One element of the stage: R(Q) (volume + surface + lift), then the
-// Adams-Bashforth commit and the positivity limiter (mode 0) or R only (mode 1).
-// k is the finest substep count of the schedule; kComp: compensated state update.
-template <typename T, int N, bool kComp = false>
-__device__ __forceinline__ void stage_element(const StageParams<T>& p, const T* __restrict__ sops, int e,
-                                              long long k, double* injected) {
-  using D = Dims<N>;
-  constexpr int NP = D::NP, NPP = D::NPP;
-  const Sched& sc = p.sc;
-  const T g = (T)p.ph.g, hvel = (T)p.ph.hvel;
-  const size_t ks = (size_t)sc.KS;
-  const size_t fstride = (size_t)NP * ks;            // between fields
-  const size_t bstride = 3 * fstride;                // between buffers
-  const int lev = level_of(sc, e);
-  const long long a = k >> (lev - 1);
-  const int src = (int)(a & 1);
-  T eta[NPP], hu[NPP], hv[NPP], bb[NPP];
-  load_nodes_m<T, NP, NPP>(p.s.q + src * bstride + 0 * fstride + e, ks, eta);
-  load_nodes_m<T, NP, NPP>(p.s.q + src * bstride + 1 * fstride + e, ks, hu);
-  load_nodes_m<T, NP, NPP>(p.s.q + src * bstride + 2 * fstride + e, ks, hv);
-  load_nodes<T, NP, NPP>(p.s.B + e, ks, bb);
-  const T rx = __ldg(p.s.geo + 4 * (size_t)e + 0), ry = __ldg(p.s.geo + 4 * (size_t)e + 1);
-  const T sx = __ldg(p.s.geo + 4 * (size_t)e + 2), sy = __ldg(p.s.geo + 4 * (size_t)e + 3);
-  // depth form of the pressure for dry elements; with inexact rules (collocation,
-  // order 2N) the pre-balanced form everywhere (the two forms then differ)
-  const T md = (Dims<N>::EXACT && ldm(p.s.dry + e)) ? T(1) : T(0);
-
-  T R0[NP], R1[NP], R2[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) { R0[i] = 0; R1[i] = 0; R2[i] = 0; }
-
-  // ---- volume term (Section 7.1): interpolate, flux + source, project ----
-  volume_term<T, N>(sops, eta, hu, hv, bb, rx, ry, sx, sy, md, g, hvel, R0, R1, R2);
-
-  auto own = [&](int f, int jn) -> T { return f == 0 ? eta[jn] : (f == 1 ? hu[jn] : (f == 2 ? hv[jn] : bb[jn])); };
-  surface_lift<T, N, false>(p, sops, e, k, own, rx, ry, sx, sy, md, R0, R1, R2);
-  add_reference_pressure<T, N>(sops, eta, bb, g, rx, ry, sx, sy, R1, R2);
-  commit_and_limit<T, N, kComp>(p, sops, e, lev, a, eta, hu, hv, bb, rx, ry, sx, sy, R0, R1, R2, injected);
-}
-
-// Elements e0, e0 + step, ... below e1 of the stage; returns the mass the
-// positivity limiter's dry resets injected (inlined by the separate launch and the
-// persistent batch kernel alike).
-template <typename T, int N, bool kComp = false>
-__device__ __forceinline__ double stage_range(const StageParams<T>& __restrict__ p, const T* __restrict__ sops,
-                                           int e0, int step, int e1, long long k) {
-  double injected = 0.0;
-  for (int e = e0; e < e1; e += step) stage_element<T, N, kComp>(p, sops, e, k, &injected);
-  return injected;
-}
-
-// kGlobalOps: the operators are read from global memory (through L1) instead of
-// the block's shared-memory copy (the operator-placement comparison of Section 7.4).
-// kComp: compensated state update (p.s.comp).
-template <typename T, int N, bool kGlobalOps = false, bool kComp = false>
-__global__ void __launch_bounds__(kBlock) k_stage(const __grid_constant__ StageParams<T> p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const T* sops;
-  if constexpr (kGlobalOps) {
-    sops = p.s.ops;
-  } else {
-    stage_ops<T, N>(reinterpret_cast<T*>(smem_raw), p.s.ops);
-    sops = reinterpret_cast<const T*>(smem_raw);
-  }
-  const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
-  double injected;
-  if constexpr (kGlobalOps) {
-    injected = 0.0;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < p.nactive; e += gridDim.x * blockDim.x)
-      stage_element<T, N>(p, sops, e, k, &injected);
-  } else {
-    injected = stage_range<T, N, kComp>(p, sops, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x,
-                                        p.nactive, k);
-  }
-  if (injected != 0.0) atomicAdd(p.s.acc, injected);
 }
 
 // --------------------------------------------------------------------------

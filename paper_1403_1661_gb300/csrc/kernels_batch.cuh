@@ -25,6 +25,7 @@
 
 #include "kernels.cuh"
 #include "kernels_tc.cuh"
+#include "kernels_team.cuh"
 
 namespace swe {
 
@@ -120,7 +121,8 @@ __global__ void __launch_bounds__(kTC ? kTcMaxBlock : kBatchTile, 1) k_batch(con
   if constexpr (kTC) {
     stage_ops<T, N, TcSmem<N>::OPS>(sops, bl.scn[0].s.ops);
   } else {
-    stage_ops<T, N>(sops, bl.scn[0].s.ops);
+    team_ops_begin<T, N>(sops, bl.scn[0].s.ops);
+    team_ops_ready();
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int total = __ldcg(&bl.ctl->total);
@@ -191,8 +193,11 @@ __global__ void __launch_bounds__(kTC ? kTcMaxBlock : kBatchTile, 1) k_batch(con
           const int t1 = min(t0 + kBatchStageTile / 32, (nactive + 31) / 32);
           injected = stage_tc_range<N>(wp, k, nactive, sops, sw, t0, 1, t1, true);
         } else {
-          const int e0 = tile * kBatchStageTile;
-          injected = stage_range<T, N>(wp, sops, e0 + lane, 32, min(e0 + kBatchStageTile, nactive), k);
+          using C = Team<T, N>;
+          T* sw = sops + C::OPS + warp * C::WARP;
+          const int t0 = tile * (kBatchStageTile / C::E);
+          const int t1 = min(t0 + kBatchStageTile / C::E, (nactive + C::E - 1) / C::E);
+          injected = team_range<T, N>(wp, sops, sops + C::PRE, sw, t0, 1, t1, nactive, k);
         }
       } else {
         const int e0 = tile * kBatchTvbTile;

@@ -3,9 +3,9 @@
 // memory (the Q^g of the update kernel, Section 7.3), the volume term by a second
 // (Section 7.1) and the surface term by a third that reads the stored traces of
 // both sides of every face (Section 7.2). R only, level-synchronous state, output
-// in the caller's layout (as swe_rhs). The arithmetic is the fused SIMT kernel's:
-// the same traces relative to the same face references, the same flux and lift;
-// only the volume and surface sums are added in the other order.
+// in the caller's layout (as swe_rhs). The traces, face references, flux and lift are the
+// fused kernel's up to rounding; the volume term keeps the weak pressure p'' and the
+// strong reference term (see the formulation in kernels.cuh).
 #pragma once
 
 #include "kernels.cuh"
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kBlock) k_split_surface(StageParams<T> p, Spli
   constexpr int NP = D::NP, NPP = D::NPP, NG = D::NG;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sops = reinterpret_cast<T*>(smem_raw);
-  stage_ops<T, N, O::TAIL>(sops, p.s.ops);
+  stage_ops<T, N>(sops, p.s.ops);
   const Sched& sc = p.sc;
   const long long k = (*p.s.macro) * (1LL << (sc.L - 1)) + p.j;
   const T g = (T)p.ph.g, hvel = (T)p.ph.hvel, hg = T(0.5) * g, qg = T(0.25) * g;

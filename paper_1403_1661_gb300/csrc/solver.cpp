@@ -341,7 +341,11 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
   };
   put_rows(O::LGT, e.Lg, 3 * ng, np, true);  // Lg is np x 3ng
   for (int g = 0; g < ng; ++g)
-    for (int m = 0; m < nfp; ++m) o[O::I1D + (size_t)g * nfpp + m] = e.I1d[(size_t)g * nfp + m];
+    for (int m = 0; m < nfp; ++m) {
+      o[O::I1D + (size_t)g * nfpp + m] = e.I1d[(size_t)g * nfp + m];
+      o[O::I1P + ((size_t)g * nfpp + m) * 2] = e.I1d[(size_t)g * nfp + m];
+      o[O::I1P + ((size_t)g * nfpp + m) * 2 + 1] = e.I1d[(size_t)(ng - 1 - g) * nfp + m];
+    }
   for (int j = 0; j < np; ++j) o[O::MW + j] = e.mean_w[j];
   for (int v = 0; v < 3; ++v)
     for (int j = 0; j < np; ++j) o[O::T1 + (size_t)v * npp + j] = e.T1[(size_t)v * np + j];
@@ -360,6 +364,26 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
       o[O::DR + (size_t)i * npp + j] = dr;
       o[O::DS + (size_t)i * npp + j] = ds;
     }
+  // mass operator of the volume term: hu, hv have degree N, so Pr (Ic hu) is one nodal
+  // product, and the projections and the lift in groups of four points
+  for (int i = 0; i < np; ++i) {
+    for (int j = 0; j < np; ++j) {
+      double wr = 0.0, ws = 0.0;
+      for (int c = 0; c < nc; ++c) {
+        wr += e.Pr[(size_t)i * nc + c] * e.Ic[(size_t)c * np + j];
+        ws += e.Ps[(size_t)i * nc + c] * e.Ic[(size_t)c * np + j];
+      }
+      o[O::WR + (size_t)i * npp + j] = wr;
+      o[O::WS + (size_t)i * npp + j] = ws;
+    }
+    for (int c = 0; c < nc; ++c) {
+      const std::vector<double>* pj[3] = {&e.Pr, &e.Ps, &e.P};
+      for (int op = 0; op < 3; ++op)
+        o[O::PROJ4 + (((size_t)(c / 4) * 3 + op) * npp + i) * 4 + c % 4] = (*pj[op])[(size_t)i * nc + c];
+    }
+    for (int q = 0; q < 3 * ng; ++q)
+      o[O::LIFT4 + ((size_t)(q / 4) * npp + i) * 4 + q % 4] = -e.Lg[(size_t)i * 3 * ng + q];
+  }
   put_rows(O::IC, e.Ic, nc, np, false);
   put_rows(O::ICR, e.Icr, nc, np, false);
   put_rows(O::ICS, e.Ics, nc, np, false);
