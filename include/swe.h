@@ -391,12 +391,13 @@ int swe_set_open_faces(swe_solver* solver, const uint8_t* open);
 int swe_set_launch_config(swe_solver* solver, int32_t ctas_per_sm);
 
 /* Warps per CTA of the tensor-core stage kernel and of the persistent batch kernel
- * (FP32 tensor-core tier; default 4, 2 at N = 5). Each warp owns its shared-memory tiles and the
- * CTA one copy of the operators, so more warps per CTA share that copy: at N = 5
- * (29 KB of tiles per warp) seven warps fit on an SM as one CTA where two CTAs of
- * four do not. warps in 1..8; SWE_EINVAL when that many warps' tiles do not fit on
- * an SM, SWE_EUNSUPPORTED on the other tiers. Used by the autotuner; results do not
- * depend on it. A batch takes the warps of the first solver of each group at
+ * (FP32 tensor-core tier; default 6 at N = 1 to 3, 4 at N = 4, 7 at N = 5). Each warp
+ * owns its shared-memory tiles and the CTA one copy of the operators, so more warps per
+ * CTA share that copy: at N = 5 (21 KB of tiles per warp, 65 KB of operators) one CTA of
+ * seven warps fits on an SM. warps in 1..8; SWE_EINVAL when that many warps' tiles do not
+ * fit on an SM, SWE_EUNSUPPORTED on the other tiers. A launch with few elements uses
+ * fewer warps per CTA, so that they spread over the SMs. Used by the autotuner; results do
+ * not depend on it. A batch takes the warps of the first solver of each group at
  * swe_batch_create. */
 int swe_set_tc_warps(swe_solver* solver, int32_t warps);
 

@@ -77,7 +77,6 @@ struct OpLayout {
 //   CT   cubature points in tiles of 8 (n of the interpolation, k of the projection)
 //   NT   nodes in tiles of 8 (n of the projection and of the lift)
 //   KF   the 3 Ng face Gauss points padded to the k8 step of the lift; KT = KF / 8
-//   FR   rows per field of the shared flux / R tile, max(KF, NPT)
 template <int N>
 struct TcDims {
   using D = Dims<N>;
@@ -88,23 +87,25 @@ struct TcDims {
   static constexpr int NPT = 8 * NT;
   static constexpr int KF = (3 * D::NG + 7) / 8 * 8;
   static constexpr int KT = KF / 8;
-  static constexpr int FR = KF > NPT ? KF : NPT;
 };
 
-// Operator fragments in register order (uint32 = two bf16), hi and lo parts.
-//   INTERP [3 ops Ic,Icr,Ics][CT][KSTEP][2 parts][32 lanes][2 regs]
-//   PROJ   [3 ops Pr,Ps,P][CT][NT][2 parts][32 lanes]
-//   LIFT   [KT][NT][2 parts][32 lanes], the B operand -L^g^T (face points x nodes)
-//   DIFF   [2 ops Dr,Ds][KP/8][NT][2 parts][32 lanes][2 regs], TF32 B operands
+// Operator fragments in register order (uint32 = two bf16, or one TF32 value), a lane's
+// words side by side.
+//   INTERP [CT][3 ops Ic,Icr,Ics][KSTEP][32 lanes][hi 2, lo 2]
+//   PROJ   [CT][NT][3 ops Pr,Ps,P][32 lanes][hi, lo]
+//   MASS   [2 ops Pr Ic, Ps Ic][KSTEP][NT][32 lanes][hi 2, lo 2]
+//   LIFT   [KT][NT][32 lanes][hi, lo], the B operand -L^g^T (face points x nodes)
+//   DIFF   [2 ops Dr,Ds][KP/8][NT][32 lanes][hi 2, lo 2], TF32 B operands
 //          Dr^T, Ds^T (nodes x nodes) of m16n8k8.tf32
 template <int N>
 struct TcLayout {
   using C = TcDims<N>;
   static constexpr int INTERP = 0;
-  static constexpr int PROJ = INTERP + 3 * C::CT * C::KSTEP * 2 * 64;
-  static constexpr int LIFT = PROJ + 3 * C::CT * C::NT * 2 * 32;
-  static constexpr int DIFF = LIFT + C::KT * C::NT * 2 * 32;
-  static constexpr int SIZE = DIFF + 2 * (C::KP / 8) * C::NT * 2 * 64;
+  static constexpr int PROJ = INTERP + C::CT * 3 * C::KSTEP * 128;
+  static constexpr int MASS = PROJ + C::CT * C::NT * 3 * 64;
+  static constexpr int LIFT = MASS + 2 * C::KSTEP * C::NT * 128;
+  static constexpr int DIFF = LIFT + C::KT * C::NT * 64;
+  static constexpr int SIZE = DIFF + 2 * (C::KP / 8) * C::NT * 128;
 };
 
 // Pointers into the caller-owned workspace. Nodal arrays are node-major
@@ -123,7 +124,8 @@ struct DevState {
   const T* vb;          // [3][KS] vertex values of Pi1 B (static)
   const T* geo;         // [K][4] rx, ry, sx, sy
   const int4* conn;     // [K] neighbour across faces 0,1,2 (kWall, kFarField); .w packs neighbour faces
-                        // (bits 0-5), TVB stencil (6-11) and "has a finer neighbour" (12)
+                        // (bits 0-5), TVB stencil (6-11), "has a finer neighbour" (12) and the
+                        // neighbours' levels minus one (13-21; the own level at a boundary face)
   const T* tvbg;        // [K][8] alpha_i, beta_i (i = 0..2)
   T* means;             // [K][4] element means (eta, hu, hv)
   uint8_t* dry;         // [K] dry flag of the latest positivity pass
@@ -153,6 +155,9 @@ struct Phys {
   double ff_h, ff_hu, ff_hv;   // far-field state of the open boundary faces (kFarField)
   float eps_f;
   int pp, dry_mode;
+  // single-precision copies: a conversion in the kernel runs on the FP64 pipe (two lanes
+  // per SM and clock) and holds its warp for 64 clocks
+  float g_f, hvel_f, ff_h_f, ff_hu_f, ff_hv_f;
 };
 
 // One scenario: its device arrays, schedule and physics. The limiter bodies read

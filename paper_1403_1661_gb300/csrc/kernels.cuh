@@ -108,14 +108,6 @@ __device__ __forceinline__ void load_row_m(const T* p, T (&o)[LEN]) {
   for (int k = 0; k < LEN / V::n; ++k) V::unpack(pv[k], &o[k * V::n]);
 }
 
-template <typename T, int LEN>
-__device__ __forceinline__ void store_row_global(T* __restrict__ p, const T (&o)[LEN]) {
-  using V = Vec16<T>;
-  typename V::type* pv = reinterpret_cast<typename V::type*>(p);
-#pragma unroll
-  for (int k = 0; k < LEN / V::n; ++k) pv[k] = V::pack(&o[k * V::n]);
-}
-
 // Node-major element access: node i of the element at p is p[i * ks]. LEN >= NP
 // registers; the padding entries read as zero.
 template <typename T, int NP, int LEN>
@@ -142,7 +134,6 @@ __device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
 
 // Cache hints: start a line's trip from memory early, without holding registers.
 // Only addresses inside live buffers are ever passed.
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Loads of the arrays the kernels write (state, Adams-Bashforth history, half-step
@@ -155,12 +146,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 template <typename T>
 __device__ __forceinline__ T ldm(const T* p) {
   return *p;
-}
-
-template <typename T, int NP, int LEN>
-__device__ __forceinline__ void load_nodes_m(const T* p, size_t ks, T (&o)[LEN]) {
-#pragma unroll
-  for (int i = 0; i < LEN; ++i) o[i] = i < NP ? ldm(p + i * ks) : T(0);
 }
 
 template <typename T>
@@ -358,140 +343,6 @@ __device__ __forceinline__ void store_p1(T* __restrict__ p1, size_t ks, const T*
   }
 }
 
-// Surface fluxes (Section 7.2) of element e: traces at the Gauss points of its
-// three faces and the well-balanced flux, scaled by sJ/J; emit(f, gq, F0, F1, F2,
-// vx, vy) receives the flux at Gauss point gq of face f and the face's (sJ/J) n. own(f, j) returns the element's
-// own field f (eta, hu, hv, B) at node j, so the caller decides whether the state
-// sits in registers or in shared memory. With kRolled the three faces run
-// through one copy of the face code (own() must then accept run-time node
-// indices); otherwise the face loop is unrolled.
-template <typename T, int N, bool kRolled, typename Own, typename Emit>
-__device__ __forceinline__ void surface_fluxes(const StageParams<T>& p, const T* __restrict__ sops, int e,
-                                               long long k, const Own& own, T rx, T ry, T sx, T sy, T md,
-                                               Emit&& emit) {
-  using D = Dims<N>;
-  using O = OpLayout<N>;
-  constexpr int NP = D::NP, NPP = D::NPP, NFP = D::NFP, NG = D::NG;
-  const Sched& sc = p.sc;
-  const T g = (T)p.ph.g, hvel = (T)p.ph.hvel, hg = T(0.5) * g, qg = T(0.25) * g;
-  const size_t ks = (size_t)sc.KS;
-  const size_t fstride = (size_t)NP * ks;
-  const size_t bstride = 3 * fstride;
-  const int4 cn = __ldg(p.s.conn + e);
-  const T E0 = own(0, 0), B0 = own(3, 0);
-#pragma unroll (kRolled ? 1 : 3)
-  for (int f = 0; f < 3; ++f) {
-    // outward normal times sJ/J from the affine factors
-    const T vxn = f == 0 ? -sx : (f == 1 ? rx + sx : -rx);
-    const T vyn = f == 0 ? -sy : (f == 1 ? ry + sy : -ry);
-    const T v2 = vxn * vxn + vyn * vyn;
-    const T iv = rsqrt_t(v2);
-    const T nx = vxn * iv, ny = vyn * iv, hs = T(0.5) * v2 * iv;
-    // Neighbour face-node values in the NEIGHBOUR's own order: its trace at this
-    // element's Gauss point gq is its own point NG-1-gq, evaluated below with the
-    // same operands in the same order as the neighbour evaluates it, relative to
-    // the same face reference (node 0 of the lower-numbered element of the pair),
-    // so both sides of a face see bit-identical traces and take the same wet/dry
-    // and velocity decisions (the mass flux stays exactly antisymmetric).
-    T ne[NFP], nu[NFP], nv[NFP], nB[NFP];
-    T Ef = E0, Bf = B0;   // face reference: the own node 0 unless the neighbour is lower
-    const int nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
-    if (nb >= 0) {
-      const int fn = (cn.w >> (2 * f)) & 3;
-      const int ln = level_of(sc, nb);
-      const long long an = k >> (ln - 1);
-      const long long pern = 1LL << (ln - 1);
-      const long long phase = k & (pern - 1);
-      // A neighbour one level coarser is always half-way through its step here; it
-      // wrote that half-step Adams-Bashforth state at its own commit.
-      const bool half = 2 * phase == pern;
-      const T* qn = half ? p.s.qmid + (size_t)nb * 3 * NPP : p.s.q + (size_t)(an & 1) * bstride + nb;
-      const size_t sn = half ? 1 : ks, sf = half ? (size_t)NPP : fstride;   // node, field strides
-#pragma unroll
-      for (int m = 0; m < NFP; ++m) {
-        const int jn = face_node_rt(Dims<N>::N, fn, m);
-        const size_t idx = (size_t)jn * sn;
-        ne[m] = ldm(qn + idx);
-        nu[m] = ldm(qn + sf + idx);
-        nv[m] = ldm(qn + 2 * sf + idx);
-        nB[m] = __ldg(p.s.B + nb + (size_t)jn * ks);
-      }
-      if (phase == 0 && nb < e) {   // an active neighbour numbered lower: its node 0
-        Ef = ldm(qn);
-        Bf = __ldg(p.s.B + nb);
-      }
-      if (phase != 0 && !half) {  // other fractions: Adams-Bashforth polynomial at t_k
-        const int depth = an + 1 < 3 ? (int)(an + 1) : 3;
-        T w[3];
-        ab_partial_weights<T>(depth, (T)phase / (T)pern, w);
-        const T dtn = level_dt(sc, ln, T(0));
-        for (int s = 0; s < depth; ++s) {
-          const T ws = dtn * w[s];
-          const T* rs = p.s.ring + (size_t)((an - s) % 3) * bstride + nb;
-#pragma unroll
-          for (int m = 0; m < NFP; ++m) {
-            const size_t idx = (size_t)face_node_rt(Dims<N>::N, fn, m) * ks;
-            ne[m] += ws * ldm(rs + idx);
-            nu[m] += ws * ldm(rs + fstride + idx);
-            nv[m] += ws * ldm(rs + 2 * fstride + idx);
-          }
-        }
-      }
-    }
-    // own face-node values relative to the face reference, read once per face
-    T oe[NFP], ou[NFP], ov[NFP], oB[NFP];
-#pragma unroll
-    for (int m = 0; m < NFP; ++m) {
-      const int jn = face_node(Dims<N>::N, f, m);
-      oe[m] = own(0, jn) - Ef;
-      ou[m] = own(1, jn);
-      ov[m] = own(2, jn);
-      oB[m] = own(3, jn) - Bf;
-    }
-    if (nb >= 0) {
-#pragma unroll
-      for (int m = 0; m < NFP; ++m) {
-        ne[m] -= Ef;
-        nB[m] -= Bf;
-      }
-    }
-    const T hf = Ef - Bf;               // depth at the face reference
-    const T dE = Ef - E0, dB = Bf - B0; // face reference relative to the element's own
-#pragma unroll 1
-    for (int gq = 0; gq < NG; ++gq) {
-      T i1[D::NFPP], i1n[D::NFPP];
-      load_row<T, D::NFPP>(sops + O::I1D + gq * D::NFPP, i1);
-      load_row<T, D::NFPP>(sops + O::I1D + (NG - 1 - gq) * D::NFPP, i1n);
-      Trace<T> tm = {0, 0, 0, 0}, tp;
-#pragma unroll
-      for (int m = 0; m < NFP; ++m) {
-        tm.e += i1[m] * oe[m];
-        tm.hu += i1[m] * ou[m];
-        tm.hv += i1[m] * ov[m];
-        tm.b += i1[m] * oB[m];
-      }
-      if (nb >= 0) {
-        tp = {0, 0, 0, 0};
-#pragma unroll
-        for (int m = 0; m < NFP; ++m) {
-          tp.e += i1n[m] * ne[m];
-          tp.hu += i1n[m] * nu[m];
-          tp.hv += i1n[m] * nv[m];
-          tp.b += i1n[m] * nB[m];
-        }
-      } else if (nb == kFarField) {  // far field: the constant state over the continued bed
-        tp = {(T)p.ph.ff_h - hf + tm.b, (T)p.ph.ff_hu, (T)p.ph.ff_hv, tm.b};
-      } else {  // reflecting wall: mirror the normal momentum
-        const T mn = tm.hu * nx + tm.hv * ny;
-        tp = {tm.e, tm.hu - T(2) * mn * nx, tm.hv - T(2) * mn * ny, tm.b};
-      }
-      T f0, f1, f2;
-      wb_flux<T>(tm, tp, hf, tm.e + dE, tm.b + dB, md, nx, ny, vxn, vyn, hs, g, hg, qg, hvel, f0, f1, f2);
-      emit(f, gq, f0, f1, f2, vxn, vyn);
-    }
-  }
-}
-
 // The reference part of the pressure and source in strong form (element
 // reference split above): R_hu -= g h0 (r_x Dr + s_x Ds)(eta - eta0),
 // R_hv -= g h0 (r_y Dr + s_y Ds)(eta - eta0), h0 = eta0 - B0 the depth at node 0.
@@ -522,154 +373,7 @@ __device__ __forceinline__ void add_reference_pressure(const T* __restrict__ sop
   }
 }
 
-// Adams-Bashforth commit (Algorithm 1) and positivity limiter (Algorithm 3) of
-// element e (mode 0), or the R output in the caller's layout (mode 1). kComp: each
-// field's increments are summed first and added to the state with the rounding
-// error of the previous update taken back (a compensated sum, p.s.comp), so the
-// single-precision state neither drifts in total mass nor accumulates its rounding
-// step after step.
-template <typename T, int N, bool kComp = false>
-__device__ __forceinline__ void commit_and_limit(const StageParams<T>& p, const T* __restrict__ sops, int e,
-                                                 int lev, long long a, T (&eta)[Dims<N>::NPP],
-                                                 T (&hu)[Dims<N>::NPP], T (&hv)[Dims<N>::NPP],
-                                                 const T (&bb)[Dims<N>::NPP], T rx, T ry, T sx, T sy,
-                                                 const T (&R0)[Dims<N>::NP], const T (&R1)[Dims<N>::NP],
-                                                 const T (&R2)[Dims<N>::NP], double* injected_acc) {
-  using D = Dims<N>;
-  constexpr int NP = D::NP, NPP = D::NPP;
-  const Sched& sc = p.sc;
-  const int K = sc.K;
-  const int dst = (int)((a + 1) & 1);
-  const size_t ks = (size_t)sc.KS;
-  const size_t fstride = (size_t)NP * ks;
-  const size_t bstride = 3 * fstride;
-  double& injected = *injected_acc;
-  if (p.mode == 1) {  // R only, caller layout
-    const int ce = p.perm[e];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      p.out[((size_t)0 * K + ce) * NP + i] = R0[i];
-      p.out[((size_t)1 * K + ce) * NP + i] = R1[i];
-      p.out[((size_t)2 * K + ce) * NP + i] = R2[i];
-    }
-    return;
-  }
-
-  // ---- Adams-Bashforth commit (Algorithm 1) ----
-  const int depth = a + 1 < 3 ? (int)(a + 1) : 3;
-  T wab[3];
-  ab_weights<T>(depth, wab);
-  const T dtl = level_dt(sc, lev, T(0));
-  const T c0 = dtl * wab[0], c1 = dtl * wab[1], c2 = dtl * wab[2];
-  T* ring = p.s.ring;
-  const size_t eo = (size_t)e;
-  store_nodes<T, NP, NP>(ring + (size_t)(a % 3) * bstride + 0 * fstride + eo, ks, R0);
-  store_nodes<T, NP, NP>(ring + (size_t)(a % 3) * bstride + 1 * fstride + eo, ks, R1);
-  store_nodes<T, NP, NP>(ring + (size_t)(a % 3) * bstride + 2 * fstride + eo, ks, R2);
-  // The same pass over the older R slots also gives the Adams-Bashforth
-  // polynomial of this step at its middle, q(t_a + dt/2) = q + dt sum_s w_s(1/2)
-  // R^(a-s) (Section 4), which an element with a finer neighbour stores for that
-  // neighbour's next substep.
-  T wh[3];
-  ab_partial_weights<T>(depth, T(0.5), wh);
-  const T m0 = dtl * wh[0], m1 = dtl * wh[1], m2 = dtl * wh[2];
-  T x0[NP], x1[NP], x2[NP];
-  T d0[kComp ? NP : 1], d1[kComp ? NP : 1], d2[kComp ? NP : 1];   // compensated: the increments
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    x0[i] = eta[i] + m0 * R0[i];
-    x1[i] = hu[i] + m0 * R1[i];
-    x2[i] = hv[i] + m0 * R2[i];
-    if constexpr (kComp) {
-      d0[i] = c0 * R0[i];
-      d1[i] = c0 * R1[i];
-      d2[i] = c0 * R2[i];
-    } else {
-      eta[i] += c0 * R0[i];
-      hu[i] += c0 * R1[i];
-      hv[i] += c0 * R2[i];
-    }
-  }
-  for (int s = 1; s < depth; ++s) {
-    const T cs = s == 1 ? c1 : c2, ms = s == 1 ? m1 : m2;
-    const T* rs = ring + (size_t)((a - s) % 3) * bstride + eo;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const T r0 = ldm(rs + i * ks), r1 = ldm(rs + fstride + i * ks);
-      const T r2 = ldm(rs + 2 * fstride + i * ks);
-      if constexpr (kComp) {
-        d0[i] += cs * r0;
-        d1[i] += cs * r1;
-        d2[i] += cs * r2;
-      } else {
-        eta[i] += cs * r0;
-        hu[i] += cs * r1;
-        hv[i] += cs * r2;
-      }
-      x0[i] += ms * r0;
-      x1[i] += ms * r1;
-      x2[i] += ms * r2;
-    }
-  }
-  if ((__ldg(reinterpret_cast<const int*>(p.s.conn + e) + 3) >> 12) & 1) {
-    T* qm = p.s.qmid + eo * 3 * NPP;
-    T row[NPP];
-#pragma unroll
-    for (int i = 0; i < NPP; ++i) row[i] = i < NP ? x0[i] : T(0);
-    store_row_global<T, NPP>(qm, row);
-#pragma unroll
-    for (int i = 0; i < NPP; ++i) row[i] = i < NP ? x1[i] : T(0);
-    store_row_global<T, NPP>(qm + NPP, row);
-#pragma unroll
-    for (int i = 0; i < NPP; ++i) row[i] = i < NP ? x2[i] : T(0);
-    store_row_global<T, NPP>(qm + 2 * NPP, row);
-  }
-  if constexpr (kComp) {
-    // q + d with the previous rounding error c taken back: y = d - c, t = q + y, and
-    // the new error c = (t - q) - y (exact when |q| >= |y|). All previous errors are
-    // read before the first new one is written, so the loads overlap.
-    T* cp = p.s.comp + eo;
-    T ce[NP], cu[NP], cv[NP];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      ce[i] = ldm(cp + i * ks);
-      cu[i] = ldm(cp + fstride + i * ks);
-      cv[i] = ldm(cp + 2 * fstride + i * ks);
-    }
-    auto add = [&](T& q, T d, T c, T* cout) {
-      const T y = d - c;
-      const T t = q + y;
-      *cout = (t - q) - y;
-      q = t;
-    };
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      add(eta[i], d0[i], ce[i], cp + i * ks);
-      add(hu[i], d1[i], cu[i], cp + fstride + i * ks);
-      add(hv[i], d2[i], cv[i], cp + 2 * fstride + i * ks);
-    }
-  }
-
-  // ---- positivity limiter (Algorithm 3) and means ----
-  T mean[3];
-  const int dryf = positivity<T, N>(eta, hu, hv, bb, sops, __ldg(p.s.Bbar + e), rx, ry, sx, sy, p.ph,
-                                    &injected, mean);
-  if (!(isfinite((double)mean[0]) && isfinite((double)mean[1]) && isfinite((double)mean[2])))
-    atomicOr(p.s.flags, 1);
-  store_nodes<T, NP, NPP>(p.s.q + dst * bstride + 0 * fstride + eo, ks, eta);
-  store_nodes<T, NP, NPP>(p.s.q + dst * bstride + 1 * fstride + eo, ks, hu);
-  store_nodes<T, NP, NPP>(p.s.q + dst * bstride + 2 * fstride + eo, ks, hv);
-  p.s.means[4 * (size_t)e + 0] = mean[0];
-  p.s.means[4 * (size_t)e + 1] = mean[1];
-  p.s.means[4 * (size_t)e + 2] = mean[2];
-  p.s.dry[e] = (uint8_t)dryf;
-  store_p1<T, N>(p.s.p1 + eo, ks, sops, eta, hu, hv);
-}
-
 // --------------------------------------------------------------------------
-// the stage kernel: R(Q) for one element (volume + surface + lift), then the
-// Adams-Bashforth commit and the positivity limiter (mode 0) or R only (mode 1)
-
 // Volume term N(Q) (Section 7.1) of one element, accumulated into R: interpolate
 // to the cubature points, volume flux and source there, project back.
 template <typename T, int N>

@@ -100,14 +100,14 @@ __device__ __forceinline__ BatchSeg load_seg(const BatchSeg* p) {
 
 // kTC: the tensor-core stage body (FP32 tier); otherwise the SIMT body (T = float
 // or double). Every warp of the CTA takes tickets on its own (no barrier in the
-// loop): a stage ticket is two warp-tiles of 32 elements, a TVB ticket 128 elements,
+// loop): a stage ticket is 64 elements (four tensor-core tiles), a TVB ticket 128 elements,
 // four to a lane. Lane 0 holds the warp's next ticket with its segment record,
 // fetched while the warp works on the current one, and waits only when a ticket
 // opens a segment it has not yet waited for (the tiles a segment needs are the same
 // for all its tickets). The warp prefetches the next stage ticket's node planes to
 // L2, as the separate launch does a tile ahead.
 template <typename T, int N, bool kTC>
-__global__ void __launch_bounds__(kTC ? kTcMaxBlock : kBatchTile, 1) k_batch(const __grid_constant__ BatchLaunch<T> bl) {
+__global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k_batch(const __grid_constant__ BatchLaunch<T> bl) {
   static_assert(kBatchStageTile % 32 == 0 && kBatchTvbTile % 32 == 0, "whole warp-tiles per ticket");
   static_assert(sizeof(BatchLaunch<T>) <= 32000, "batch launch parameters exceed the kernel-parameter space");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -119,7 +119,9 @@ __global__ void __launch_bounds__(kTC ? kTcMaxBlock : kBatchTile, 1) k_batch(con
   // every scenario of the group has the same operators: stage the first one's
   // (the staging ends with a CTA barrier, which also publishes s_k0)
   if constexpr (kTC) {
-    stage_ops<T, N, TcSmem<N>::OPS>(sops, bl.scn[0].s.ops);
+    tc_ops_begin<N>(sops, bl.scn[0].s.ops, bl.scn[0].s.tcops);
+    stage_tc_init<N>(sops + TcSmem<N>::CTA + (threadIdx.x >> 5) * TcSmem<N>::WARP);
+    team_ops_ready();
   } else {
     team_ops_begin<T, N>(sops, bl.scn[0].s.ops);
     team_ops_ready();
@@ -188,10 +190,11 @@ __global__ void __launch_bounds__(kTC ? kTcMaxBlock : kBatchTile, 1) k_batch(con
       double injected = 0.0;
       if (kind == 0) {
         if constexpr (kTC) {
-          float* sw = sops + TcSmem<N>::OPS + warp * TcSmem<N>::WARP;
-          const int t0 = tile * (kBatchStageTile / 32);
-          const int t1 = min(t0 + kBatchStageTile / 32, (nactive + 31) / 32);
-          injected = stage_tc_range<N>(wp, k, nactive, sops, sw, t0, 1, t1, true);
+          using SM = TcSmem<N>;
+          float* sw = sops + SM::CTA + warp * SM::WARP;
+          const int t0 = tile * (kBatchStageTile / SM::E);
+          const int t1 = min(t0 + kBatchStageTile / SM::E, (nactive + SM::E - 1) / SM::E);
+          injected = stage_tc_range<N>(wp, k, nactive, sops, sw, t0, 1, t1, true, false);
         } else {
           using C = Team<T, N>;
           T* sw = sops + C::OPS + warp * C::WARP;

@@ -254,18 +254,20 @@ __global__ void k_gather_rows(const E* __restrict__ src, E* __restrict__ dst, in
   }
 }
 
-// connectivity in the new order: neighbours renumbered, "has a finer neighbour"
-// (bit 12 of .w) recomputed from the new levels
+// connectivity in the new order: neighbours renumbered, "has a finer neighbour" (bit 12
+// of .w) and the neighbours' levels (bits 13-21) recomputed from the new levels
 __global__ void k_remap_conn(const int4* __restrict__ src, int4* __restrict__ dst, int K, const int* __restrict__ pi,
                              const int* __restrict__ sigma, const uint8_t* __restrict__ lev_new) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < K; e += gridDim.x * blockDim.x) {
     int4 c = src[pi[e]];
     int nb[3] = {c.x, c.y, c.z};
-    int w = c.w & ~(1 << 12);
+    int w = c.w & 0xfff;
     for (int f = 0; f < 3; ++f) {
-      if (nb[f] < 0) continue;
-      nb[f] = sigma[nb[f]];
-      if (lev_new[nb[f]] < lev_new[e]) w |= 1 << 12;
+      if (nb[f] >= 0) {
+        nb[f] = sigma[nb[f]];
+        if (lev_new[nb[f]] < lev_new[e]) w |= 1 << 12;
+      }
+      w |= (lev_new[nb[f] >= 0 ? nb[f] : e] - 1) << (13 + 3 * f);
     }
     dst[e] = make_int4(nb[0], nb[1], nb[2], w);
   }

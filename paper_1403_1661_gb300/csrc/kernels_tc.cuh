@@ -2,42 +2,59 @@
 // tier with split-BF16 products, Section 7.1's N(Q) = Pr cF1 + Ps cF2 + P cS and
 // Section 7.2's R = N - L^g F).
 //
-// Each warp owns 32 elements (two 16-row m-tiles). First one thread per element
-// computes the face traces and well-balanced fluxes at its 3 Ng Gauss points
-// (shared with the SIMT kernel) into the warp's shared flux tile. Then per m-tile
-// and per tile of 8 cubature points:
-//   interpolation  D[16 el x 8 pts] = State[16 el x Np] * Op^T  (mma m16n8k16),
-//                  for eta, hu, hv, B with Ic and for B with Icr, Ics;
-//   flux           evaluated in registers on the accumulator layout: lane (g, t)
-//                  holds elements g, g+8 at cubature points 2t, 2t+1, which is
-//                  exactly the A-fragment layout of the next product;
-//   projection     R[16 el x Np] += Flux[16 el x 8 pts] * Pr^T (Ps^T, P^T)
-//                  (mma m16n8k8), accumulated over all cubature tiles;
-// and, on the same accumulators, per tile of 8 face points
-//   lift           R[16 el x Np] -= SurfaceFlux[16 el x 8 pts] * L^g^T (m16n8k8).
-// Every product is split: a = a_hi + a_lo in bfloat16 (operators and data), and
-// a*b ~ a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with FP32 accumulation (relative error
-// of order 2^-16 per product). The warp then hands R and the state to one thread
-// per element through shared memory for the Adams-Bashforth commit and the
-// positivity limiter, which are shared with the SIMT kernel.
+// A warp holds a tile of 16 elements, one row of the m16 products each. Phases:
+//   surface   lane (el, half): faces 0 and 1 one per lane, then face 2 with its Gauss
+//             points shared by the two lanes of the element: traces and well-balanced
+//             fluxes (team_flux) into the warp's flux tile
+//   lift      R[16 el x Np] -= Flux[16 el x 8 pts] * L^g^T, 8 face points at a time
+//   split     the state relative to node 0 as BF16 pairs hi + lo into the tile the
+//             fluxes occupied, where ldmatrix reads it as A fragments
+//   volume    per tile of 8 cubature points: interpolation (m16n8k16) of h, hu, hv with
+//             Ic and eta with Icr, Ics; the flux on the accumulator layout, where lane
+//             (g, t) holds rows g, g + 8 at points 2t, 2t + 1, which is the A layout of
+//             the next product; projection with Pr, Ps, P (k16 instructions, two of the
+//             split products side by side in k)
+//   mass      R_h += rx WR hu + ry WR hv + sx WS hu + sy WS hv (nodal operators)
+//   reference -g h0 (r_x Dr + s_x Ds) eta, the leading term at depth, in TF32 splits
+//   commit    lane (el, half), half of the nodes each: team_commit
+// Every BF16 product is split: a = a_hi + a_lo (operators and data) and
+// a b ~ a_hi b_hi + a_hi b_lo + a_lo b_hi with FP32 accumulation (relative error of
+// order 2^-16); TF32 splits 2^-21. The volume term is the form of kernels_team.cuh: with
+// exact rules -P[g (h - h0) grad eta] carries pressure and source, h0 the depth at node 0
+// (its product with grad eta is the reference term); the other schemes keep p'' and
+// -g eta' grad B'.
+//
+// The operators' fragments are staged once per CTA in shared memory; results do not
+// depend on the number of warps per CTA.
+//
+// What bounds it: latency at two to three warps per scheduler (no pipe is above 25 %,
+// shared memory at half of its wavefronts; more warps cost the registers or the L1 that
+// the gathers need). Per 32 elements at N = 4 it issues 8.5 k warp instructions where
+// the form with 32-element tiles, six interpolated rows, eight projected fluxes and
+// unpacked arithmetic took 11.8 k. Sixteen elements per tile, so that a small active set
+// has twice the tiles and each takes half the time. Measured (GB300), before and after:
+//   one R, 500,000 elements, N = 4                            0.340 -> 0.242 ms
+//   45,149 elements, N = 3, 25 macro steps with transfers      6.39 -> 5.25 ms
+//   2,048 elements, N = 2, 6 macro steps with transfers        0.964 -> 0.788 ms
 #pragma once
 
 #include <cuda_bf16.h>
 
 #include "kernels.cuh"
+#include "kernels_team.cuh"
 
 namespace swe {
 
-constexpr int kTcWarps = 4;                  // warps per CTA unless a solver sets another count
-constexpr int kTcBlock = 32 * kTcWarps;
-constexpr int kTcMaxWarps = 8;               // 8 warps x 32 threads x 255 registers fill the register file
-constexpr int kTcMaxBlock = 32 * kTcMaxWarps;
-
-__device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  mma_k16(d, a[0], a[1], a[2], a[3], b0, b1);
 }
 
 __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
@@ -53,6 +70,13 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void ldmatrix4(uint32_t (&a)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+               : "r"(addr)
+               : "memory");
+}
+
 // float -> (hi, lo) TF32 pair: hi rounded to 10 mantissa bits, lo the remainder
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
@@ -60,474 +84,550 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
 }
 
 // two floats -> (hi, lo) bf16x2 pairs; the first float goes to the low half
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-  const float2 hf = __bfloat1622float2(h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - hf.x, x1 - hf.y);
+__device__ __forceinline__ void split2(float2 x, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
   hi = *reinterpret_cast<const uint32_t*>(&h);
+  const float2 hf = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+  const float2 r = add2(x, make_float2(-hf.x, -hf.y));
+  const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// Per-warp shared tiles are node-major with the 32 elements of the warp
-// contiguous and a stride of LS = 36 words per node: one thread per element
-// reads a node of its own element without bank conflicts, and the mma fragment
-// reads (rows g, g+8, nodes 2t, 2t+1) land on 32 distinct banks.
-constexpr int LS = 36;
+// Per-warp shared tiles. State, fluxes and R are node-major with the 16 elements
+// contiguous and LS = 20 words per node: the mma fragment reads (rows g, g+8; nodes or
+// points 2t, 2t+1) land on 32 distinct banks. The BF16 tile holds rows of KP values (one
+// element) 2 KP + 16 bytes apart, so the eight row addresses of an ldmatrix cover all
+// banks.
+constexpr int LS = 20;
 
 template <int N>
 struct TcSmem {
   using D = Dims<N>;
   using C = TcDims<N>;
-  // per warp: state [4 fields][KP nodes][LS]; surface fluxes [3][KF face points][LS],
-  // later R [3][NPT nodes][LS] in the same rows (field stride FR); geo [32][4];
-  // pressure form md [32]
+  static constexpr int E = 16;                            // elements per warp-tile
+  static constexpr int BS = C::KP / 2 + 4;                // words per row of the BF16 tile
+  static constexpr int mx(int a, int b) { return a > b ? a : b; }
+  // per warp: state [4 fields][KP nodes][LS]; then, one after the other in the same
+  // words, surface fluxes [3][KF][LS], the BF16 tile [4 fields][hi, lo][16][BS] and R
+  // [3][NPT][LS]; geometry [16][4]
   static constexpr int STATE = 0;
-  static constexpr int FRT = STATE + 4 * C::KP * LS;
-  static constexpr int GEO = FRT + 3 * C::FR * LS;
-  static constexpr int MD = GEO + 32 * 4;
-  static constexpr int WARP = MD + 32;                   // floats per warp
-  static constexpr int OPS = OpLayout<N>::TAIL;          // floats of per-element operators (staged first)
-  // dynamic shared memory of a CTA of `warps` warps: one operator copy, one tile set per warp
-  static constexpr int bytes(int warps) { return (OPS + warps * WARP) * 4; }
-  static constexpr int BYTES = bytes(kTcWarps);
+  static constexpr int TILE = STATE + 4 * C::KP * LS;
+  static constexpr int GEO = TILE + mx(mx(3 * C::KF * LS, 4 * 2 * E * BS), 3 * C::NPT * LS);
+  static constexpr int WARP = GEO + E * 4;                // floats per warp
+  static constexpr int OPS = OpLayout<N>::TAIL;           // floats of per-element operators
+  static constexpr int FRAG = OPS;                        // then the operator fragments
+  static constexpr int CTA = OPS + TcLayout<N>::SIZE;     // floats per CTA before the warps' tiles
+  // dynamic shared memory of a CTA of `warps` warps
+  static constexpr int bytes(int warps) { return (CTA + warps * WARP) * 4; }
+  // warps per SM the registers are budgeted for, as many as a CTA may have: twelve up to
+  // N = 3 (168 registers), eight at N = 4 (255; twelve spill), seven at N = 5 (their
+  // tiles and the fragments fill the shared memory)
+  static constexpr int LIMIT = D::N <= 3 ? 12 : (D::N == 4 ? 8 : 7);
+  // default warps per CTA (ms per macro step of a 125k-element beach, 45k at N = 5):
+  // N = 2 0.206 (four 0.204, twelve 0.220), N = 3 0.334 (four 0.358, twelve 0.338),
+  // N = 4 0.363 (eight 0.371, two 0.375), N = 5 0.374 (six 0.375, four 0.433)
+  static constexpr int WARPS = D::N <= 3 ? 6 : (D::N == 4 ? 4 : 7);
 };
 
-// One warp-tile of 32 elements (element e = 32 tile + lane): load, surface fluxes,
-// volume term and lift on tensor cores, commit and limiter. k: the finest substep
-// count of the schedule; nactive: elements [0, nactive) are active at this substep;
-// next_tile: the warp's next tile (its planes are prefetched to L2), or -1; sw: the
-// warp's shared tiles; kComp: compensated state update in the commit.
+// One warp-tile of 16 elements (element e = 16 tile + el). k: the finest substep count;
+// nactive: elements [0, nactive) are active at this substep; next_tile: the warp's next
+// tile (its planes are prefetched to L2), or -1; first: the CTA's operators are still on
+// their way; sops: per-element operators followed by the fragments; sw: the warp's tiles;
+// kComp: compensated state update in the commit.
 template <int N, bool kComp = false>
 __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long long k, int nactive,
-                                              const float* sops, float* sw, int tile, int next_tile,
-                                              double* injected) {
+                                              const float* sops, float* sw, int tile, int ntiles, int next_tile,
+                                              bool first, double* injected) {
   using D = Dims<N>;
   using C = TcDims<N>;
   using TL = TcLayout<N>;
   using SM = TcSmem<N>;
-  constexpr int NP = D::NP, NPP = D::NPP, KP = C::KP, KSTEP = C::KSTEP, CT = C::CT, NT = C::NT;
-  constexpr int NG = D::NG, KT = C::KT, KF = C::KF, FR = C::FR;
-  // operator fragments stay in global memory: every warp reads the same few KB,
-  // which the L1 cache serves
-  const uint32_t* __restrict__ stc = p.s.tcops;
+  constexpr int NP = D::NP, NPP = D::NPP, NFP = D::NFP, KP = C::KP, KSTEP = C::KSTEP, CT = C::CT, NT = C::NT;
+  constexpr bool kBothFaces = D::N == 4;   // registers for both faces' gathers at once
+  constexpr int NG = D::NG, KT = C::KT, KF = C::KF, NPT = C::NPT, NB = NPP / 2, BS = SM::BS;
+  const uint32_t* sfrag = reinterpret_cast<const uint32_t*>(sops) + SM::FRAG;
   const int lane = threadIdx.x & 31;
+  const int el = lane & 15, half = lane >> 4;
   const int g = lane >> 2, t = lane & 3;
-  float* s_state = sw + SM::STATE;
-  float* s_FR = sw + SM::FRT;
-  float* s_geo = sw + SM::GEO;
-  float* s_md = sw + SM::MD;
+  float* st = sw + SM::STATE;
+  float* sx = sw + SM::TILE;
   const Sched& sc = p.sc;
-  const float gg = (float)p.ph.g, hvel = (float)p.ph.hvel, hg = 0.5f * gg;
-  const size_t ks = (size_t)sc.KS, fstride = (size_t)NP * ks, bstride = 3 * fstride;
-  // ---- load: lane = element; each node plane is one coalesced 128-byte line ----
-  const int e = tile * 32 + lane;
-  const bool valid = e < nactive;
-  int lev = 1;
-  long long a = 0;
-  if (valid) {
-    lev = level_of(sc, e);
-    a = k >> (lev - 1);
-    const float* qe = p.s.q + (size_t)(a & 1) * bstride + e;
+  const float gg = p.ph.g_f, hvel = p.ph.hvel_f;
+  const size_t fstride = (size_t)NP * sc.KS, bstride = 3 * fstride;
+  // lanes past the last active element repeat it (and store nothing)
+  const bool valid = tile < ntiles && tile * 16 + el < nactive;
+  const int e = valid ? tile * 16 + el : nactive - 1;
+  const int lev = level_of(sc, e);
+  const long long a = k >> (lev - 1);
+  float4 ge;
+
+  // ---- gather: the own nodes (half of them per lane), the first face's neighbour ----
+  TeamFace<float, NFP> fc, fc2;   // the lane's first face, and face 2
+  bool finer = false;
+  {
+    float own[4][NB];
+    if (tile < ntiles) {
+      const int4 cn = __ldg(p.s.conn + e);
+      finer = (cn.w >> 12) & 1;
+      team_load_face<float, N>(p, cn, e, half, k, fc);
+      if (kBothFaces) team_load_face<float, N>(p, cn, e, 2, k, fc2);
+      const unsigned ks4 = (unsigned)sc.KS, o0 = half * NB * ks4;
+      const float* q0 = p.s.q + (size_t)(a & 1) * bstride + e + o0;
+      const float *q1 = q0 + fstride, *q2 = q1 + fstride, *qb = p.s.B + e + o0;
 #pragma unroll
-    for (int f = 0; f < 3; ++f)
+      for (int n = 0; n < NB; ++n) {
+        if (NB + n < NP || half * NB + n < NP) {
+          own[0][n] = ldm(q0 + n * ks4);
+          own[1][n] = ldm(q1 + n * ks4);
+          own[2][n] = ldm(q2 + n * ks4);
+          own[3][n] = __ldg(qb + n * ks4);
+        }
+      }
+      ge = __ldg(reinterpret_cast<const float4*>(p.s.geo) + e);
+    }
+    // this tile's older R slots and the next tile's planes start moving now (hints; the
+    // first element's level stands for the tile)
+    if (p.mode == 0 && tile < ntiles) {
+      const int e0 = tile * 16;
+      const long long a0 = __shfl_sync(0xffffffffu, a, 0);
+      const int s0 = ring_slot3(a0);
+      const float* ra = p.s.ring + (size_t)(s0 == 0 ? 2 : s0 - 1) * bstride + e0;
+      const float* rb = p.s.ring + (size_t)(s0 == 2 ? 0 : s0 + 1) * bstride + e0;
 #pragma unroll
-      for (int i = 0; i < NP; ++i) s_state[(f * KP + i) * LS + lane] = ldm(qe + f * fstride + i * ks);
+      for (int pl = 0; pl < 3 * NP; pl += 32)
+        if (pl + lane < 3 * NP) {
+          const unsigned o = (unsigned)(pl + lane) * (unsigned)sc.KS;
+          prefetch_l2(ra + o);
+          prefetch_l2(rb + o);
+          if constexpr (kComp) prefetch_l2(p.s.comp + e0 + o);
+        }
+    }
+    if (next_tile >= 0 && next_tile * 16 < nactive) {
+      const int e0 = next_tile * 16;
+      const long long an = k >> (level_of(sc, e0) - 1);
+      const float* qn = p.s.q + (size_t)(an & 1) * bstride + e0;
+      const float* bn = p.s.B + e0;
 #pragma unroll
-    for (int i = 0; i < NP; ++i) s_state[(3 * KP + i) * LS + lane] = __ldg(p.s.B + e + i * ks);
-    reinterpret_cast<float4*>(s_geo)[lane] = __ldg(reinterpret_cast<const float4*>(p.s.geo) + e);
-    // depth form of the pressure for dry elements (exact rules only)
-    s_md[lane] = (Dims<N>::EXACT && ldm(p.s.dry + e)) ? 1.f : 0.f;
-  } else {
-    s_md[lane] = 0.f;
+      for (int pl = 0; pl < 3 * NP; pl += 32)
+        if (pl + lane < 3 * NP) prefetch_l2(qn + (unsigned)(pl + lane) * (unsigned)sc.KS);
+      if (lane < NP) prefetch_l2(bn + (unsigned)lane * (unsigned)sc.KS);
+    }
+    if (first) team_ops_ready();
+    if (tile >= ntiles) return;
 #pragma unroll
     for (int f = 0; f < 4; ++f)
 #pragma unroll
-      for (int i = 0; i < NP; ++i) s_state[(f * KP + i) * LS + lane] = 0.f;
-    reinterpret_cast<float4*>(s_geo)[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-#pragma unroll
-  for (int f = 0; f < 4; ++f)
-#pragma unroll
-    for (int i = NP; i < KP; ++i) s_state[(f * KP + i) * LS + lane] = 0.f;
-  __syncwarp();
-
-  // the next tile's planes and this tile's older R slots start moving now: one
-  // 128-byte line per lane and plane (the parity of the first element stands for
-  // the tile; these are hints, every address lies inside its array)
-  {
-    const int e0n = next_tile * 32;
-    if (next_tile >= 0 && e0n < nactive) {
-      const long long an = k >> (level_of(sc, e0n) - 1);
-      const float* qn = p.s.q + (size_t)(an & 1) * bstride + e0n;
-      for (int pl = lane; pl < 4 * NP; pl += 32)
-        prefetch_l2(pl < 3 * NP ? qn + pl * ks : p.s.B + e0n + (pl - 3 * NP) * ks);
-    }
-    const long long a0 = __shfl_sync(0xffffffffu, a, 0);
-    if (p.mode == 0) {
-      const int e0 = tile * 32;
-      for (int s = 1; s < 3 && s <= a0; ++s) {
-        const float* rs = p.s.ring + (size_t)((a0 - s) % 3) * bstride + e0;
-        for (int pl = lane; pl < 3 * NP; pl += 32) prefetch_l2(rs + pl * ks);
-      }
-      if constexpr (kComp)
-        for (int pl = lane; pl < 3 * NP; pl += 32) prefetch_l2(p.s.comp + e0 + pl * ks);
-    }
-  }
-
-  // ---- surface fluxes, one thread per element, into the warp's flux tile ----
-  {
-    float* sf = s_FR + lane;
-    for (int q = 3 * NG; q < KF; ++q) {  // padding points: zero rows for the lift
-      sf[(0 * FR + q) * LS] = 0.f;
-      sf[(1 * FR + q) * LS] = 0.f;
-      sf[(2 * FR + q) * LS] = 0.f;
-    }
-    if (valid) {
-      const float4 ge = reinterpret_cast<const float4*>(s_geo)[lane];
-      const float* my = s_state + lane;
-      auto own = [&](int f, int jn) -> float { return my[(f * KP + jn) * LS]; };
-      // the element's node-0 flux, subtracted here and from the volume fluxes (see
-      // the reference flux below): constant fluxes contribute nothing to R
-      const float hu0 = my[(1 * KP) * LS], hv0 = my[(2 * KP) * LS], d0 = my[0] - my[(3 * KP) * LS];
-      const float id0 = d0 > hvel ? recip(d0) : 0.f;
-      const float u0 = hu0 * id0, v0 = hv0 * id0;
-      surface_fluxes<float, N, true>(p, sops, e, k, own, ge.x, ge.y, ge.z, ge.w, s_md[lane],
-                                     [&](int f, int gq, float f0, float f1, float f2, float vx, float vy) {
-                                       const int q = f * NG + gq;
-                                       const float fr = hu0 * vx + hv0 * vy;
-                                       sf[(0 * FR + q) * LS] = f0 - fr;
-                                       sf[(1 * FR + q) * LS] = f1 - u0 * fr;
-                                       sf[(2 * FR + q) * LS] = f2 - v0 * fr;
-                                     });
-    } else {
-      for (int q = 0; q < 3 * NG; ++q) {
-        sf[(0 * FR + q) * LS] = 0.f;
-        sf[(1 * FR + q) * LS] = 0.f;
-        sf[(2 * FR + q) * LS] = 0.f;
-      }
-    }
+      for (int n = 0; n < NB; ++n)
+        if (NB + n < NP || half * NB + n < NP) st[(f * KP + half * NB + n) * LS + el] = own[f][n];
+    if (half == 0) reinterpret_cast<float4*>(sw + SM::GEO)[el] = ge;
   }
   __syncwarp();
 
-  // ---- volume term and lift on tensor cores, one m-tile of 16 elements at a time ----
+  // ---- surface fluxes into the tile ----
+  {
+    for (int q = 3 * NG + half; q < KF; q += 2)   // padding points: zero rows for the lift
+      sx[(0 * KF + q) * LS + el] = sx[(1 * KF + q) * LS + el] = sx[(2 * KF + q) * LS + el] = 0.f;
+    const float* my = st + el;
+    const float E0 = my[0], B0 = my[3 * KP * LS];
+    // the element's node-0 flux, subtracted here and from the volume fluxes (a constant
+    // flux adds nothing to R), so the split products see only the variation
+    const float hu0 = my[KP * LS], hv0 = my[2 * KP * LS], d0 = E0 - B0;
+    const float id0 = d0 > hvel ? recip_fast(d0) : 0.f;
+    const float u0 = hu0 * id0, v0 = hv0 * id0;
 #pragma unroll 1
-  for (int mt = 0; mt < 2; ++mt) {
-    const int r0 = 16 * mt + g, r1 = r0 + 8;
-    // State A fragments (rows r0, r1; nodes 16ks + {2t, 2t+1, 2t+8, 2t+9}), hi and
-    // lo. The surface and the bed enter relative to their values at node 0 of the
-    // element (eta0, B0): the interpolation of a constant is exact and its
-    // derivatives vanish (Ic B = B0 + Ic (B - B0), Icr B = Icr (B - B0)), so only
-    // the within-element variation carries the split-product error, whether the
-    // bed is thousands of metres deep or the water a millimetre thin.
-    // All four fields enter relative to their node-0 values (c0 for row r0, c1 for r1).
-    float c0[4], c1[4];
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      c0[f] = s_state[(f * KP) * LS + r0];
-      c1[f] = s_state[(f * KP) * LS + r1];
-    }
-    const float cE0 = c0[0], cE1 = c1[0], cB0 = c0[3], cB1 = c1[3];
-    uint32_t ah[4][KSTEP][4], al[4][KSTEP][4];
-#pragma unroll
-    for (int f = 0; f < 4; ++f)
-#pragma unroll
-      for (int ks = 0; ks < KSTEP; ++ks) {
-        const float* sn = s_state + (f * KP + 16 * ks + 2 * t) * LS;   // node 16ks + 2t
-        const float d0 = c0[f], d1 = c1[f];
-        const float2 v00 = make_float2(sn[r0] - d0, sn[LS + r0] - d0);
-        const float2 v10 = make_float2(sn[r1] - d1, sn[LS + r1] - d1);
-        const float2 v01 = make_float2(sn[8 * LS + r0] - d0, sn[9 * LS + r0] - d0);
-        const float2 v11 = make_float2(sn[8 * LS + r1] - d1, sn[9 * LS + r1] - d1);
-        split2(v00.x, v00.y, ah[f][ks][0], al[f][ks][0]);
-        split2(v10.x, v10.y, ah[f][ks][1], al[f][ks][1]);
-        split2(v01.x, v01.y, ah[f][ks][2], al[f][ks][2]);
-        split2(v11.x, v11.y, ah[f][ks][3], al[f][ks][3]);
+    for (int r = 0; r < 2; ++r) {
+      const int f = r == 0 ? half : 2;
+      const int g0 = r == 0 || half == 0 ? 0 : (NG + 1) / 2, g1 = r == 0 || half == 1 ? NG : (NG + 1) / 2;
+      if (r == 1) {
+        if (kBothFaces) fc = fc2;
+        else team_load_face<float, N>(p, __ldg(p.s.conn + e), e, 2, k, fc);
       }
-    const float4 ge0 = reinterpret_cast<const float4*>(s_geo)[r0];
-    const float4 ge1 = reinterpret_cast<const float4*>(s_geo)[r1];
-    // Reference flux: the volume fluxes cF1, cF2 of each row's node-0 state. A
-    // constant flux adds nothing to R (its volume term and its own-side lift
-    // cancel exactly), so it is subtracted here and from the surface fluxes and
-    // the split products see only the flux's variation over the element (the
-    // pressure p'' vanishes at node 0).
-    float fr0[6], fr1[6];
-    {
-      const float d0 = cE0 - cB0, d1 = cE1 - cB1;
-      const float i0 = d0 > hvel ? recip(d0) : 0.f, i1v = d1 > hvel ? recip(d1) : 0.f;
-      const float u0 = c0[1] * i0, v0 = c0[2] * i0, u1 = c1[1] * i1v, v1 = c1[2] * i1v;
-      const float a0r = ge0.x * c0[1] + ge0.y * c0[2], b0r = ge0.z * c0[1] + ge0.w * c0[2];
-      const float a1r = ge1.x * c1[1] + ge1.y * c1[2], b1r = ge1.z * c1[1] + ge1.w * c1[2];
-      fr0[0] = a0r; fr0[1] = u0 * a0r; fr0[2] = v0 * a0r; fr0[3] = b0r; fr0[4] = u0 * b0r; fr0[5] = v0 * b0r;
-      fr1[0] = a1r; fr1[1] = u1 * a1r; fr1[2] = v1 * a1r; fr1[3] = b1r; fr1[4] = u1 * b1r; fr1[5] = v1 * b1r;
-    }
-    float Racc[3][NT][4];
+      const float Ef = fc.lower ? fc.E : E0, Bf = fc.lower ? fc.B : B0;
+      float vx, vy;
+      face_normal(f, ge.x, ge.y, ge.z, ge.w, vx, vy);
+      const float v2 = mad(vx, vx, vy * vy), iv = rsqrt_fast(v2);
+      const float nx = vx * iv, ny = vy * iv, hs = 0.5f * v2 * iv;
+      float2 tr[NFP][4];   // (own, neighbour) relative to the face reference
 #pragma unroll
-    for (int f = 0; f < 3; ++f)
+      for (int m = 0; m < NFP; ++m) {
+        const float* o = my + face_node_rt(D::N, f, m) * LS;
+        tr[m][0] = add2(make_float2(o[0], fc.v[0][m]), dup(-Ef));
+        tr[m][1] = make_float2(o[KP * LS], fc.v[1][m]);
+        tr[m][2] = make_float2(o[2 * KP * LS], fc.v[2][m]);
+        tr[m][3] = add2(make_float2(o[3 * KP * LS], fc.v[3][m]), dup(-Bf));
+      }
+      const float fr = mad(hu0, vx, hv0 * vy), fu = u0 * fr, fv = v0 * fr;
+#pragma unroll 1
+      for (int gq = g0; gq < g1; ++gq) {
+        const float* w = sops + OpLayout<N>::I1P + 2 * gq * D::NFPP;
+        float2 te = dup(0.f), tu = te, tv = te, tb = te;
+#pragma unroll
+        for (int m = 0; m < NFP; m += 2) {
+          float2 wp[2];
+          load4(w + 2 * m, wp);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            if (m + c >= NFP) continue;
+            te = fma2(wp[c], tr[m + c][0], te);
+            tu = fma2(wp[c], tr[m + c][1], tu);
+            tv = fma2(wp[c], tr[m + c][2], tv);
+            tb = fma2(wp[c], tr[m + c][3], tb);
+          }
+        }
+        float f0, f1, f2;
+        team_flux<float, N>(p.ph, fc.nb, Ef, Bf, E0, B0, nx, ny, hs, vx, vy, te, tu, tv, tb, f0, f1, f2);
+        float* o = sx + (f * NG + gq) * LS + el;
+        o[0] = f0 - fr;
+        o[KF * LS] = f1 - fu;
+        o[2 * KF * LS] = f2 - fv;
+      }
+    }
+  }
+  __syncwarp();
+
+  // ---- lift: R -= Flux * L^g^T, k8 tiles of 8 face points ----
+  const int r0 = g, r1 = g + 8;
+  float Racc[3][NT][4];
+#pragma unroll
+  for (int f = 0; f < 3; ++f)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) Racc[f][nt][c] = 0.f;
+#pragma unroll
+  for (int kt = 0; kt < KT; ++kt) {
+    uint2 lb[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+      lb[nt] = reinterpret_cast<const uint2*>(sfrag + TL::LIFT)[(kt * NT + nt) * 32 + lane];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      const float* fq = sx + (f * KF + 8 * kt + 2 * t) * LS;
+      uint32_t ah0, al0, ah1, al1;
+      split2(make_float2(fq[r0], fq[LS + r0]), ah0, al0);
+      split2(make_float2(fq[r1], fq[LS + r1]), ah1, al1);
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        mma_k16(Racc[f][nt], al0, al1, ah0, ah1, lb[nt].x, lb[nt].y);   // lo hi + hi lo
+        mma_k8(Racc[f][nt], ah0, ah1, lb[nt].x);
+      }
+    }
+  }
+  __syncwarp();   // every lane has read the fluxes before the BF16 tile overwrites them
+
+  // ---- split: the state relative to node 0 (h' or eta', hu', hv', eta' or B') ----
+  {
+    constexpr int KH = KP / 2;   // nodes per lane, padding included
+    const float* my = st + el;
+    float c0[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) c0[f] = my[f * KP * LS];
+    uint32_t* bt = reinterpret_cast<uint32_t*>(sx) + el * BS + half * (KH / 2);
+#pragma unroll
+    for (int j = 0; j < KH; j += 8) {
+      uint32_t hi[4][4], lo[4][4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        // nodes half * KH + j + 2c, + 1; those past NP meet zero operator entries, so any
+        // finite value will do (their rows hold zeros)
+        const float* o = my + (half * KH + j + 2 * c) * LS;
+        float2 v[4];
+        if (j + 2 * c >= NP) {   // past NP in both halves
+#pragma unroll
+          for (int f = 0; f < 4; ++f) v[f] = make_float2(0.f, 0.f);
+        } else {
+          float2 x[4];
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+            x[f] = add2(make_float2(o[f * KP * LS], o[(f * KP + 1) * LS]), dup(-c0[f]));
+          v[0] = D::EXACT ? add2(x[0], make_float2(-x[3].x, -x[3].y)) : x[0];
+          v[1] = x[1];
+          v[2] = x[2];
+          v[3] = D::EXACT ? x[0] : x[3];
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) split2(v[f], hi[f][c], lo[f][c]);
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        *reinterpret_cast<uint4*>(bt + (2 * f) * 16 * BS + j / 2) = make_uint4(hi[f][0], hi[f][1], hi[f][2], hi[f][3]);
+        *reinterpret_cast<uint4*>(bt + (2 * f + 1) * 16 * BS + j / 2) =
+            make_uint4(lo[f][0], lo[f][1], lo[f][2], lo[f][3]);
+      }
+    }
+  }
+  __syncwarp();
+  // ldmatrix address of this lane: row (lane & 15), k offset 8 (lane >> 4)
+  const uint32_t bt0 = (uint32_t)__cvta_generic_to_shared(sx) + ((lane & 15) * BS + (lane >> 4) * 4) * 4;
+  auto afrag = [&](int f, int part, int ks, uint32_t (&o)[4]) {
+    ldmatrix4(o, bt0 + ((2 * f + part) * 16 * BS + ks * 8) * 4);
+  };
+
+  const float4 ge0 = reinterpret_cast<const float4*>(sw + SM::GEO)[r0];
+  const float4 ge1 = reinterpret_cast<const float4*>(sw + SM::GEO)[r1];
+  const float cE0 = st[r0], cE1 = st[r1];
+  // ---- mass: X = W (hu', hv') per nodal operator, combined with the affine factors ----
+#pragma unroll
+  for (int f = 1; f < 3; ++f) {
+    float X[2][NT][4];
+#pragma unroll
+    for (int op = 0; op < 2; ++op)
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) Racc[f][nt][c] = 0.f;
+        for (int c = 0; c < 4; ++c) X[op][nt][c] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < KSTEP; ++ks) {
+      uint32_t ah[4], al[4];
+      afrag(f, 0, ks, ah);
+      afrag(f, 1, ks, al);
+#pragma unroll
+      for (int op = 0; op < 2; ++op)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          const uint4 b = reinterpret_cast<const uint4*>(sfrag + TL::MASS)[((op * KSTEP + ks) * NT + nt) * 32 + lane];
+          mma_k16(X[op][nt], al, b.x, b.y);
+          mma_k16(X[op][nt], ah, b.z, b.w);
+          mma_k16(X[op][nt], ah, b.x, b.y);
+        }
+    }
+    const float wr0 = f == 1 ? ge0.x : ge0.y, wr1 = f == 1 ? ge1.x : ge1.y;
+    const float ws0 = f == 1 ? ge0.z : ge0.w, ws1 = f == 1 ? ge1.z : ge1.w;
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        Racc[0][nt][c] =
+            mad(c < 2 ? ws0 : ws1, X[1][nt][c], mad(c < 2 ? wr0 : wr1, X[0][nt][c], Racc[0][nt][c]));
+  }
 
-    // interpolation fragments of the first cubature tile
-    uint2 ibh[3][KSTEP], ibl[3][KSTEP];
+  // ---- volume: 8 cubature points at a time ----
+  {
+    const float2 hu0 = make_float2(st[KP * LS + r0], st[KP * LS + r1]);
+    const float2 hv0 = make_float2(st[2 * KP * LS + r0], st[2 * KP * LS + r1]);
+    const float2 h0 = make_float2(cE0 - st[3 * KP * LS + r0], cE1 - st[3 * KP * LS + r1]);
+    float fr[2][4];   // the momentum fluxes of node 0, per row
 #pragma unroll
-    for (int op = 0; op < 3; ++op)
-#pragma unroll
-      for (int ks = 0; ks < KSTEP; ++ks) {
-        const uint32_t* fb = stc + TL::INTERP + (((op * CT + 0) * KSTEP + ks) * 2) * 64 + lane * 2;
-        ibh[op][ks] = __ldg(reinterpret_cast<const uint2*>(fb));
-        ibl[op][ks] = __ldg(reinterpret_cast<const uint2*>(fb + 64));
-      }
+    for (int r = 0; r < 2; ++r) {
+      const float h = r ? h0.y : h0.x, mu = r ? hu0.y : hu0.x, mv = r ? hv0.y : hv0.x;
+      const float4 ger = r ? ge1 : ge0;
+      const float ih = h > hvel ? recip_fast(h) : 0.f;
+      const float a0 = mad(ger.x, mu, ger.y * mv), b0 = mad(ger.z, mu, ger.w * mv);
+      fr[r][0] = mu * ih * a0;
+      fr[r][1] = mv * ih * a0;
+      fr[r][2] = mu * ih * b0;
+      fr[r][3] = mv * ih * b0;
+    }
 #pragma unroll 1
     for (int ct = 0; ct < CT; ++ct) {
-      // projection fragments of this tile: in flight during the interpolation and flux
-      uint32_t pbh[3][NT], pbl[3][NT];
+      constexpr int NA = D::EXACT ? 5 : 6;   // h', hu', hv', eta_r, eta_s; or eta', hu', hv', B_r, B_s, B'
+      float acc[NA][4];
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int op = 0; op < 3; ++op) {
-          const uint32_t* fb = stc + TL::PROJ + (((op * CT + ct) * NT + nt) * 2) * 32 + lane;
-          pbh[op][nt] = __ldg(fb);
-          pbl[op][nt] = __ldg(fb + 32);
-        }
-      // interpolation: acc[0..3] = (eta, hu, hv, B) * Ic, acc[4] = B * Icr, acc[5] = B * Ics
-      float acc[6][4];
-#pragma unroll
-      for (int o = 0; o < 6; ++o)
+      for (int o = 0; o < NA; ++o)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[o][c] = 0.f;
 #pragma unroll
       for (int ks = 0; ks < KSTEP; ++ks) {
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          mma_k16(acc[f], al[f][ks], ibh[0][ks].x, ibh[0][ks].y);
-          mma_k16(acc[f], ah[f][ks], ibl[0][ks].x, ibl[0][ks].y);
-          mma_k16(acc[f], ah[f][ks], ibh[0][ks].x, ibh[0][ks].y);
-        }
-#pragma unroll
-        for (int op = 1; op < 3; ++op) {
-          mma_k16(acc[3 + op], al[3][ks], ibh[op][ks].x, ibh[op][ks].y);
-          mma_k16(acc[3 + op], ah[3][ks], ibl[op][ks].x, ibl[op][ks].y);
-          mma_k16(acc[3 + op], ah[3][ks], ibh[op][ks].x, ibh[op][ks].y);
-        }
-      }
-      // interpolation fragments of the next tile: in flight during the flux and projection
-      if (ct + 1 < CT) {
-#pragma unroll
-        for (int op = 0; op < 3; ++op)
-#pragma unroll
-          for (int ks = 0; ks < KSTEP; ++ks) {
-            const uint32_t* fb = stc + TL::INTERP + (((op * CT + ct + 1) * KSTEP + ks) * 2) * 64 + lane * 2;
-            ibh[op][ks] = __ldg(reinterpret_cast<const uint2*>(fb));
-            ibl[op][ks] = __ldg(reinterpret_cast<const uint2*>(fb + 64));
-          }
-      }
-      // flux and source at the lane's four points: (r0, 2t), (r0, 2t+1), (r1, 2t), (r1, 2t+1)
-      float fl[8][4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float4 ge = c < 2 ? ge0 : ge1;
-        const float rx = ge.x, ry = ge.y, sx = ge.z, sy = ge.w;
-        // eta - eta0 and B - B0 at the point (element reference split)
-        const float ec = acc[0][c];
-        const float huc = (c < 2 ? c0[1] : c1[1]) + acc[1][c], hvc = (c < 2 ? c0[2] : c1[2]) + acc[2][c];
-        const float bpc = acc[3][c];
-        const float brc = acc[4][c], bsc = acc[5][c];
-        const float hc = (c < 2 ? cE0 - cB0 : cE1 - cB1) + (ec - bpc);
-        const float ih = hc > hvel ? recip(hc) : 0.f;
-        const float u = huc * ih, v = hvc * ih;
-        // momentum rows of cF1, cF2 written through the mass row; p'' (the
-        // reference part is added in strong form before the commit)
-        const float md = c < 2 ? s_md[r0] : s_md[r1];
-        const float ep = ec - md * bpc;
-        const float pr = hg * ep * (ec - (2.f - md) * bpc);
-        const float a0 = rx * huc + ry * hvc, b0 = sx * huc + sy * hvc;
-        const float* fr = c < 2 ? fr0 : fr1;
-        fl[0][c] = a0 - fr[0];
-        fl[1][c] = (u * a0 + rx * pr) - fr[1];
-        fl[2][c] = (v * a0 + ry * pr) - fr[2];
-        fl[3][c] = b0 - fr[3];
-        fl[4][c] = (u * b0 + sx * pr) - fr[4];
-        fl[5][c] = (v * b0 + sy * pr) - fr[5];
-        const float gm = -gg * ep;
-        fl[6][c] = gm * (rx * brc + sx * bsc);
-        fl[7][c] = gm * (ry * brc + sy * bsc);
-      }
-      // A fragments (m16n8k8): reg0 = row r0 (points 2t, 2t+1), reg1 = row r1
-      uint32_t fh[8][2], flo[8][2];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        split2(fl[q][0], fl[q][1], fh[q][0], flo[q][0]);
-        split2(fl[q][2], fl[q][3], fh[q][1], flo[q][1]);
-      }
-      // projection: R_h += cF1_h Pr + cF2_h Ps; R_m += cF1_m Pr + cF2_m Ps + cS_m P
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const uint32_t bh[3] = {pbh[0][nt], pbh[1][nt], pbh[2][nt]};
-        const uint32_t bl[3] = {pbl[0][nt], pbl[1][nt], pbl[2][nt]};
+        const uint4* ib = reinterpret_cast<const uint4*>(sfrag + TL::INTERP) + ((ct * 3) * KSTEP + ks) * 32 + lane;
+        const uint4 b0 = ib[0], b1 = ib[KSTEP * 32], b2 = ib[2 * KSTEP * 32];
+        uint32_t ah[4], al[4];
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
-          // cF1 (quantity f) with Pr, cF2 (3+f) with Ps, source (5+f, f>0) with P
-          mma_k8(Racc[f][nt], flo[f][0], flo[f][1], bh[0]);
-          mma_k8(Racc[f][nt], fh[f][0], fh[f][1], bl[0]);
-          mma_k8(Racc[f][nt], fh[f][0], fh[f][1], bh[0]);
-          mma_k8(Racc[f][nt], flo[3 + f][0], flo[3 + f][1], bh[1]);
-          mma_k8(Racc[f][nt], fh[3 + f][0], fh[3 + f][1], bl[1]);
-          mma_k8(Racc[f][nt], fh[3 + f][0], fh[3 + f][1], bh[1]);
-          if (f > 0) {
-            mma_k8(Racc[f][nt], flo[5 + f][0], flo[5 + f][1], bh[2]);
-            mma_k8(Racc[f][nt], fh[5 + f][0], fh[5 + f][1], bl[2]);
-            mma_k8(Racc[f][nt], fh[5 + f][0], fh[5 + f][1], bh[2]);
-          }
+          afrag(f, 0, ks, ah);
+          afrag(f, 1, ks, al);
+          mma_k16(acc[f], al, b0.x, b0.y);
+          mma_k16(acc[f], ah, b0.z, b0.w);
+          mma_k16(acc[f], ah, b0.x, b0.y);
+        }
+        afrag(3, 0, ks, ah);
+        afrag(3, 1, ks, al);
+        mma_k16(acc[3], al, b1.x, b1.y);
+        mma_k16(acc[4], al, b2.x, b2.y);
+        mma_k16(acc[3], ah, b1.z, b1.w);
+        mma_k16(acc[4], ah, b2.z, b2.w);
+        mma_k16(acc[3], ah, b1.x, b1.y);
+        mma_k16(acc[4], ah, b2.x, b2.y);
+        if constexpr (!D::EXACT) {
+          mma_k16(acc[NA - 1], al, b0.x, b0.y);
+          mma_k16(acc[NA - 1], ah, b0.z, b0.w);
+          mma_k16(acc[NA - 1], ah, b0.x, b0.y);
         }
       }
-    }
-    // lift: R -= Flux * L^g^T over the face points, k8 tiles of 8 points; the
-    // fluxes of rows r0, r1 at points 8kt + 2t, 2t + 1 form the A fragments
+      // flux and source at the lane's four points, a row (two points) at a time:
+      // 0..3 the advective momentum fluxes (Pr hu, hv; Ps hu, hv), 4, 5 the source
+      uint32_t fh[6][2], fl[6][2];
 #pragma unroll
-    for (int kt = 0; kt < KT; ++kt) {
-      uint32_t lbh[NT], lbl[NT];
+      for (int r = 0; r < 2; ++r) {
+        const float4 ger = r ? ge1 : ge0;
+        auto at = [&](int o) { return make_float2(acc[o][2 * r], acc[o][2 * r + 1]); };
+        const float2 rx = dup(ger.x), ry = dup(ger.y), sxv = dup(ger.z), sy = dup(ger.w);
+        const float2 mu = add2(dup(r ? hu0.y : hu0.x), at(1)), mv = add2(dup(r ? hv0.y : hv0.x), at(2));
+        const float2 dh = D::EXACT ? at(0) : add2(at(0), make_float2(-acc[NA - 1][2 * r], -acc[NA - 1][2 * r + 1]));
+        const float2 hc = add2(dup(r ? h0.y : h0.x), dh);
+        const float2 ih = make_float2(hc.x > hvel ? recip_fast(hc.x) : 0.f, hc.y > hvel ? recip_fast(hc.y) : 0.f);
+        const float2 u = mul2(mu, ih), v = mul2(mv, ih);
+        const float2 am = fma2(rx, mu, mul2(ry, mv)), bm = fma2(sxv, mu, mul2(sy, mv));
+        const float2 dr = at(3), ds = at(4);
+        float2 F[6];
+        if constexpr (D::EXACT) {
+          F[0] = fma2(u, am, dup(-fr[r][0]));
+          F[1] = fma2(v, am, dup(-fr[r][1]));
+          F[2] = fma2(u, bm, dup(-fr[r][2]));
+          F[3] = fma2(v, bm, dup(-fr[r][3]));
+        } else {
+          const float2 ec = at(0), bc = at(NA - 1);
+          const float2 pr = mul2(mul2(dup(0.5f * gg), ec), fma2(dup(-2.f), bc, ec));
+          F[0] = fma2(u, am, fma2(rx, pr, dup(-fr[r][0])));
+          F[1] = fma2(v, am, fma2(ry, pr, dup(-fr[r][1])));
+          F[2] = fma2(u, bm, fma2(sxv, pr, dup(-fr[r][2])));
+          F[3] = fma2(v, bm, fma2(sy, pr, dup(-fr[r][3])));
+        }
+        const float2 gm = mul2(dup(-gg), D::EXACT ? dh : at(0));
+        F[4] = mul2(gm, fma2(rx, dr, mul2(sxv, ds)));
+        F[5] = mul2(gm, fma2(ry, dr, mul2(sy, ds)));
+#pragma unroll
+        for (int q = 0; q < 6; ++q) split2(F[q], fh[q][r], fl[q][r]);
+      }
+      // projection: R_hu += Pr F0 + Ps F2 + P F4, R_hv += Pr F1 + Ps F3 + P F5; the nine
+      // split products of a field go in pairs through the k16 instruction
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        const uint32_t* fb = stc + TL::LIFT + ((kt * NT + nt) * 2) * 32 + lane;
-        lbh[nt] = __ldg(fb);
-        lbl[nt] = __ldg(fb + 32);
-      }
+        const uint2* pb = reinterpret_cast<const uint2*>(sfrag + TL::PROJ) + ((ct * NT + nt) * 3) * 32 + lane;
+        const uint2 pr = pb[0], ps = pb[32], pp = pb[64];   // (hi, lo)
 #pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        const float* fq = s_FR + (f * FR + 8 * kt + 2 * t) * LS;
-        uint32_t ah0, al0, ah1, al1;
-        split2(fq[r0], fq[LS + r0], ah0, al0);
-        split2(fq[r1], fq[LS + r1], ah1, al1);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          mma_k8(Racc[f][nt], al0, al1, lbh[nt]);
-          mma_k8(Racc[f][nt], ah0, ah1, lbl[nt]);
-          mma_k8(Racc[f][nt], ah0, ah1, lbh[nt]);
+        for (int f = 0; f < 2; ++f) {
+          float(&R)[4] = Racc[1 + f][nt];
+          mma_k16(R, fl[f][0], fl[f][1], fl[2 + f][0], fl[2 + f][1], pr.x, ps.x);
+          mma_k16(R, fl[4 + f][0], fl[4 + f][1], fh[f][0], fh[f][1], pp.x, pr.y);
+          mma_k16(R, fh[2 + f][0], fh[2 + f][1], fh[4 + f][0], fh[4 + f][1], ps.y, pp.y);
+          mma_k16(R, fh[f][0], fh[f][1], fh[2 + f][0], fh[2 + f][1], pr.x, ps.x);
+          mma_k8(R, fh[4 + f][0], fh[4 + f][1], pp.x);
         }
       }
     }
-    // strong-form reference pressure (element reference split, see kernels.cuh):
-    // R_hu -= g h0 (rx Dr + sx Ds)(eta - eta0), R_hv -= g h0 (ry Dr + sy Ds)(eta - eta0).
-    // The leading term of R at depth, so TF32 split products (2^-21 per product).
+    // ---- reference term: R_hu -= g h0 (rx Dr + sx Ds)(eta - eta0), R_hv alike ----
     {
-      float Dacc[2][NT][4];
+      const float gh0 = -gg * h0.x, gh1 = -gg * h0.y;
+      float X[2][NT][4];
 #pragma unroll
       for (int op = 0; op < 2; ++op)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) Dacc[op][nt][c] = 0.f;
+          for (int c = 0; c < 4; ++c) X[op][nt][c] = 0.f;
 #pragma unroll
       for (int kk = 0; kk < KP / 8; ++kk) {
-        const float* sn = s_state + (8 * kk + t) * LS;   // eta at node 8kk + t
-        uint32_t eh[4], el[4];
-        split_tf32(sn[r0] - cE0, eh[0], el[0]);
-        split_tf32(sn[r1] - cE1, eh[1], el[1]);
-        split_tf32(sn[4 * LS + r0] - cE0, eh[2], el[2]);
-        split_tf32(sn[4 * LS + r1] - cE1, eh[3], el[3]);
+        const float* sn = st + (8 * kk + t) * LS;   // eta at node 8kk + t
+        uint32_t eh[4], elo[4];
+        split_tf32(sn[r0] - cE0, eh[0], elo[0]);
+        split_tf32(sn[r1] - cE1, eh[1], elo[1]);
+        split_tf32(sn[4 * LS + r0] - cE0, eh[2], elo[2]);
+        split_tf32(sn[4 * LS + r1] - cE1, eh[3], elo[3]);
 #pragma unroll
         for (int op = 0; op < 2; ++op)
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
-            const uint32_t* fb = stc + TL::DIFF + (((op * (KP / 8) + kk) * NT + nt) * 2) * 64 + lane * 2;
-            const uint2 bh = __ldg(reinterpret_cast<const uint2*>(fb));
-            const uint2 bl = __ldg(reinterpret_cast<const uint2*>(fb + 64));
-            mma_tf32(Dacc[op][nt], el, bh.x, bh.y);
-            mma_tf32(Dacc[op][nt], eh, bl.x, bl.y);
-            mma_tf32(Dacc[op][nt], eh, bh.x, bh.y);
+            const uint4 b = reinterpret_cast<const uint4*>(sfrag + TL::DIFF)[((op * (KP / 8) + kk) * NT + nt) * 32 + lane];
+            mma_tf32(X[op][nt], elo, b.x, b.y);
+            mma_tf32(X[op][nt], eh, b.z, b.w);
+            mma_tf32(X[op][nt], eh, b.x, b.y);
           }
       }
-      const float gh0 = -gg * (cE0 - cB0), gh1 = -gg * (cE1 - cB1);
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const float4 ge = c < 2 ? ge0 : ge1;
+          const float4 gc = c < 2 ? ge0 : ge1;
           const float gh = c < 2 ? gh0 : gh1;
-          Racc[1][nt][c] += gh * (ge.x * Dacc[0][nt][c] + ge.z * Dacc[1][nt][c]);
-          Racc[2][nt][c] += gh * (ge.y * Dacc[0][nt][c] + ge.w * Dacc[1][nt][c]);
+          Racc[1][nt][c] = mad(gh, mad(gc.x, X[0][nt][c], gc.z * X[1][nt][c]), Racc[1][nt][c]);
+          Racc[2][nt][c] = mad(gh, mad(gc.y, X[0][nt][c], gc.w * X[1][nt][c]), Racc[2][nt][c]);
         }
     }
-    // every lane has read this m-tile's flux columns before R overwrites them
-    __syncwarp();
-    // R of this m-tile to shared memory: rows r0, r1, nodes 8nt + {2t, 2t+1}
-#pragma unroll
-    for (int f = 0; f < 3; ++f)
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        float* rn = s_FR + (f * FR + 8 * nt + 2 * t) * LS;
-        rn[r0] = Racc[f][nt][0];
-        rn[LS + r0] = Racc[f][nt][1];
-        rn[r1] = Racc[f][nt][2];
-        rn[LS + r1] = Racc[f][nt][3];
-      }
   }
+  __syncwarp();   // the BF16 tile is read before R overwrites it
+#pragma unroll
+  for (int f = 0; f < 3; ++f)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      float* rn = sx + (f * NPT + 8 * nt + 2 * t) * LS;
+      rn[r0] = Racc[f][nt][0];
+      rn[LS + r0] = Racc[f][nt][1];
+      rn[r1] = Racc[f][nt][2];
+      rn[LS + r1] = Racc[f][nt][3];
+    }
   __syncwarp();
 
-  // ---- one thread per element: commit, positivity ----
-  if (valid) {
-    float R0[NP], R1[NP], R2[NP];
+  // ---- commit and positivity, two lanes per element ----
+  {
+    float R[3][NB], q[4][NB];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      R0[i] = s_FR[(0 * FR + i) * LS + lane];
-      R1[i] = s_FR[(1 * FR + i) * LS + lane];
-      R2[i] = s_FR[(2 * FR + i) * LS + lane];
-    }
-    const float4 ge = reinterpret_cast<const float4*>(s_geo)[lane];
-    // the per-element operators were staged at the start of shared memory with the
-    // OpLayout offsets, so the shared epilogue indexes them directly
-    const float* my = s_state + lane;
-    float eta[NPP], hu[NPP], hv[NPP], bb[NPP];
+    for (int n = 0; n < NB; ++n) {
+      const int i = half * NB + n;
 #pragma unroll
-    for (int i = 0; i < NPP; ++i) {
-      eta[i] = my[(0 * KP + i) * LS];
-      hu[i] = my[(1 * KP + i) * LS];
-      hv[i] = my[(2 * KP + i) * LS];
-      bb[i] = my[(3 * KP + i) * LS];
+      for (int f = 0; f < 3; ++f) R[f][n] = NB + n < NPT ? sx[(f * NPT + i) * LS + el] : 0.f;   // zero past NP
+#pragma unroll
+      for (int f = 0; f < 4; ++f) q[f][n] = st[(f * KP + i) * LS + el];
     }
-    commit_and_limit<float, N, kComp>(p, sops, e, lev, a, eta, hu, hv, bb, ge.x, ge.y, ge.z, ge.w, R0, R1, R2,
-                               injected);
+    team_commit<float, N, 2, NB, kComp>(p, sops, valid, finer, e, half, lev, a, q, R, ge.x, ge.y, ge.z, ge.w, injected);
   }
+  __syncwarp();   // the tiles are read before the next gather overwrites them
+}
+
+// The state rows past NP are read by the TF32 products (with zero operator entries):
+// zeroed once, never written again.
+template <int N>
+__device__ __forceinline__ void stage_tc_init(float* sw) {
+  using C = TcDims<N>;
+  constexpr int pad = (C::KP - Dims<N>::NP) * LS;
+  for (int f = 0; f < 4; ++f)
+    for (int i = threadIdx.x & 31; i < pad; i += 32) sw[(f * C::KP + Dims<N>::NP) * LS + i] = 0.f;
   __syncwarp();
 }
 
-// Warp-tiles t0, t0 + step, ... below t1 (each warp calls it for its own tiles;
-// with prefetch the planes of the warp's next tile are prefetched to L2); returns
-// the mass the positivity limiter's dry resets injected. The separate launch and
-// the persistent batch kernel both inline it (out of line the body ran 1.5 times
-// slower: its parameters become memory loads).
+// Warp-tiles t0, t0 + step, ... below t1 (each warp calls it for its own tiles; with
+// prefetch the planes of the warp's next tile are prefetched to L2); returns the mass
+// the positivity limiter's dry resets injected. The separate launch and the persistent
+// batch kernel both inline it (out of line the body ran 1.5 times slower: its parameters
+// become memory loads).
 template <int N, bool kComp = false>
 __device__ __forceinline__ double stage_tc_range(const StageParams<float>& __restrict__ p, long long k,
                                               int nactive, const float* __restrict__ sops, float* sw, int t0,
-                                              int step, int t1, bool prefetch) {
+                                              int step, int t1, bool prefetch, bool first) {
   double injected = 0.0;
-  for (int tile = t0; tile < t1; tile += step)
-    stage_tc_warp<N, kComp>(p, k, nactive, sops, sw, tile, prefetch ? tile + step : -1, &injected);
+  int tile = t0;
+  do {   // the first pass waits for the operators whether or not the warp has a tile
+    stage_tc_warp<N, kComp>(p, k, nactive, sops, sw, tile, t1, prefetch ? tile + step : -1, first, &injected);
+    first = false;
+    tile += step;
+  } while (tile < t1);
   return injected;
 }
 
-// CTA: blockDim.x / 32 warps (1 to kTcMaxWarps), each with its own shared tiles after
-// the CTA's operator copy. kComp: compensated state update (p.s.comp).
-template <int N, bool kComp = false>
-__global__ void __launch_bounds__(kTcMaxBlock, 1) k_stage_tc(const __grid_constant__ StageParams<float> p) {
+// Start the copy of a CTA's operators and fragments to shared memory.
+template <int N>
+__device__ __forceinline__ void tc_ops_begin(float* smem, const float* ops, const uint32_t* frag) {
   using SM = TcSmem<N>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* sops = reinterpret_cast<float*>(smem_raw);                       // [0, OPS)
-  {
-    const float4* src = reinterpret_cast<const float4*>(p.s.ops);
-    float4* dst = reinterpret_cast<float4*>(sops);
-    for (int i = threadIdx.x; i < SM::OPS / 4; i += blockDim.x) dst[i] = __ldg(src + i);
-    __syncthreads();
-  }
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float* sw = sops + SM::OPS + warp * SM::WARP;
-  const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
-  const int ntiles = (p.nactive + 31) / 32;
-  const double injected =
-      stage_tc_range<N, kComp>(p, k, p.nactive, sops, sw, blockIdx.x * nw + warp, gridDim.x * nw, ntiles, true);
-  if (injected != 0.0) atomicAdd(p.s.acc, injected);
+  team_copy<float, SM::OPS>(smem, ops);
+  team_copy<float, TcLayout<N>::SIZE>(smem + SM::FRAG, reinterpret_cast<const float*>(frag));
+  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+// CTA: blockDim.x / 32 warps (1 to MAXW), each with its own shared tiles after the CTA's
+// operators. kComp: compensated state update (p.s.comp).
+template <int N, bool kComp = false>
+__global__ void __launch_bounds__(32 * TcSmem<N>::LIMIT, 1) k_stage_tc(const __grid_constant__ StageParams<float> p) {
+  using SM = TcSmem<N>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* sops = reinterpret_cast<float*>(smem_raw);
+  tc_ops_begin<N>(sops, p.s.ops, p.s.tcops);
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  float* sw = sops + SM::CTA + warp * SM::WARP;
+  stage_tc_init<N>(sw);
+  const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
+  const int ntiles = (p.nactive + SM::E - 1) / SM::E;
+  const double injected =
+      stage_tc_range<N, kComp>(p, k, p.nactive, sops, sw, blockIdx.x * nw + warp, gridDim.x * nw, ntiles, true, true);
+  if (injected != 0.0) atomicAdd(p.s.acc, injected);
+}
 
 }  // namespace swe

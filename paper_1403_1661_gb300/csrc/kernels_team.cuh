@@ -83,9 +83,35 @@ __device__ __forceinline__ auto hsum(P a) { return a.x + a.y; }
 // separate launch and the batch kernel would round differently.
 __device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+// Hardware reciprocal and inverse square root without the scaling that the plain calls
+// spend on subnormal arguments (three more instructions each): depths above the dry
+// threshold and squared speeds are normal numbers. FP64: the correctly rounded ones.
+__device__ __forceinline__ float recip_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double recip_fast(double x) { return 1.0 / x; }
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt_t(x); }
 // |u| + sqrt(x), x >= 0 (FP32: the square root as in sqrt_nn)
-__device__ __forceinline__ float speed(float u, float x) { return mad(x, rsqrtf(fmaxf(x, 1e-30f)), fabsf(u)); }
+__device__ __forceinline__ float speed(float u, float x) { return mad(x, rsqrt_fast(fmaxf(x, 1e-30f)), fabsf(u)); }
 __device__ __forceinline__ double speed(double u, double x) { return fabs(u) + sqrt(x); }
+
+__device__ __forceinline__ float phys_g(const Phys& ph, float) { return ph.g_f; }
+__device__ __forceinline__ double phys_g(const Phys& ph, double) { return ph.g; }
+__device__ __forceinline__ float phys_hvel(const Phys& ph, float) { return ph.hvel_f; }
+__device__ __forceinline__ double phys_hvel(const Phys& ph, double) { return ph.hvel; }
+__device__ __forceinline__ float phys_ff(const Phys& ph, int c, float) {
+  return c == 0 ? ph.ff_h_f : (c == 1 ? ph.ff_hu_f : ph.ff_hv_f);
+}
+__device__ __forceinline__ double phys_ff(const Phys& ph, int c, double) {
+  return c == 0 ? ph.ff_h : (c == 1 ? ph.ff_hu : ph.ff_hv);
+}
 
 // four consecutive values (16-byte aligned) as two pairs
 __device__ __forceinline__ void load4(const float* p, float2 (&o)[2]) {
@@ -103,8 +129,8 @@ __device__ __forceinline__ void load4(const double* p, double2 (&o)[2]) {
 // ten FP64 instructions, and the FP64 pipe, two lanes wide per SM, is what bounds
 // that tier); symmetric in the sides, so both elements of a face get the same values.
 __device__ __forceinline__ void recip_both(float hm, float hp, float hvel, float& im, float& ip) {
-  im = hm > hvel ? recip(hm) : 0.f;
-  ip = hp > hvel ? recip(hp) : 0.f;
+  im = hm > hvel ? recip_fast(hm) : 0.f;
+  ip = hp > hvel ? recip_fast(hp) : 0.f;
 }
 __device__ __forceinline__ void recip_both(double hm, double hp, double hvel, double& im, double& ip) {
   const bool wm = hm > hvel, wp = hp > hvel;
@@ -187,53 +213,61 @@ __device__ __forceinline__ void team_ops_begin(T* smem, const T* gops) {
 template <typename T>
 struct TeamLane {
   int e, lev;
-  bool valid;
+  bool valid, finer;
   long long a;
   T rx, ry, sx, sy;
 };
 
-// The neighbour of face `part` as the lane of that face sees it: its face nodes in its
-// own order (surface_fluxes in kernels.cuh says why) and the pair's face reference.
+// The neighbour of a face as the lane of that face sees it: its face nodes in the
+// NEIGHBOUR's own order (its trace at this element's Gauss point g is its own point
+// NG-1-g, evaluated with the same operands in the same order as the neighbour evaluates
+// it) and the pair's face reference, node 0 of the lower-numbered element. Both sides of
+// a face then see bit-identical traces and take the same wet/dry and velocity decisions,
+// and the mass flux is exactly antisymmetric.
 template <typename T, int NFP>
 struct TeamFace {
   int nb;          // neighbour, kWall or kFarField
   T v[4][NFP];     // eta, hu, hv, B
-  T E, B;          // the neighbour's node 0 where it is the face reference
-  bool lower;
+  bool lower;      // the face reference is the neighbour's node 0
+  T E, B;          // then its values
 };
 
 template <typename T, int N>
-__device__ __forceinline__ void team_load_face(const StageParams<T>& p, int e, int f, long long k,
+__device__ __forceinline__ void team_load_face(const StageParams<T>& p, const int4& cn, int e, int f, long long k,
                                                TeamFace<T, Dims<N>::NFP>& o) {
   using D = Dims<N>;
   constexpr int NP = D::NP, NPP = D::NPP, NFP = D::NFP;
   const Sched& sc = p.sc;
   const size_t ks = (size_t)sc.KS, fstride = (size_t)NP * ks, bstride = 3 * fstride;
-  const int4 cn = __ldg(p.s.conn + e);
-  const int nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
-  o.nb = nb;
-  if (nb < 0) return;
+  o.nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
+  // across a boundary face the lane reads its own element: the values are replaced by the
+  // ghost state, and no lane needs a select
+  const int nb = o.nb < 0 ? e : o.nb;
   const int fn = (cn.w >> (2 * f)) & 3;
-  const int ln = level_of(sc, nb);
+  const int ln = ((cn.w >> (13 + 3 * f)) & 7) + 1;
   const long long an = k >> (ln - 1);
   const long long pern = 1LL << (ln - 1);
   const long long phase = k & (pern - 1);
   const bool half = 2 * phase == pern;   // the half-step record of a coarser neighbour
   const T* qn = half ? p.s.qmid + (size_t)nb * 3 * NPP : p.s.q + (size_t)(an & 1) * bstride + nb;
-  const size_t sn = half ? 1 : ks, sf = half ? (size_t)NPP : fstride;
+  // 32-bit node offsets (NP KS words of a plane set are always below 2^32 here: the
+  // workspace of a larger mesh would not fit the card), one wide add per access
+  const unsigned sn = half ? 1u : (unsigned)sc.KS;
+  const size_t sf = half ? (size_t)NPP : fstride;
+  const T *q1 = qn + sf, *q2 = q1 + sf, *qb = p.s.B + nb;
 #pragma unroll
   for (int m = 0; m < NFP; ++m) {
-    const int jn = face_node_rt(D::N, fn, m);
-    const size_t idx = (size_t)jn * sn;
+    const unsigned jn = (unsigned)face_node_rt(D::N, fn, m);
+    const unsigned idx = jn * sn;
     o.v[0][m] = ldm(qn + idx);
-    o.v[1][m] = ldm(qn + sf + idx);
-    o.v[2][m] = ldm(qn + 2 * sf + idx);
-    o.v[3][m] = __ldg(p.s.B + nb + (size_t)jn * ks);
+    o.v[1][m] = ldm(q1 + idx);
+    o.v[2][m] = ldm(q2 + idx);
+    o.v[3][m] = __ldg(qb + jn * (unsigned)sc.KS);
   }
-  if (phase == 0 && nb < e) {
-    o.lower = true;
+  o.lower = phase == 0 && nb < e;
+  if (o.lower) {
     o.E = ldm(qn);
-    o.B = __ldg(p.s.B + nb);
+    o.B = __ldg(qb);
   }
   if (phase != 0 && !half) {   // other fractions: Adams-Bashforth polynomial at t_k
     const int depth = an + 1 < 3 ? (int)(an + 1) : 3;
@@ -261,13 +295,13 @@ template <typename T, int N>
 __device__ __forceinline__ void team_flux(const Phys& ph, int kind, T Ef, T Bf, T E0, T B0, T nx, T ny, T hs, T vx,
                                           T vy, Pair<T> te, Pair<T> tu, Pair<T> tv, Pair<T> tb, T& f0, T& f1, T& f2) {
   using D = Dims<N>;
-  const T g = (T)ph.g, hvel = (T)ph.hvel, qg = T(0.25) * g;
+  const T g = phys_g(ph, T(0)), hvel = phys_hvel(ph, T(0)), qg = T(0.25) * g;
   const T hf = Ef - Bf;
   if (kind < 0) {
     if (kind == kFarField) {   // the constant state over the continued bed
-      te.y = (T)ph.ff_h - hf + tb.x;
-      tu.y = (T)ph.ff_hu;
-      tv.y = (T)ph.ff_hv;
+      te.y = phys_ff(ph, 0, T(0)) - hf + tb.x;
+      tu.y = phys_ff(ph, 1, T(0));
+      tv.y = phys_ff(ph, 2, T(0));
     } else {                   // reflecting wall: mirror the normal momentum
       const T mn = T(-2) * mad(tu.x, nx, tv.x * ny);
       te.y = te.x;
@@ -319,22 +353,20 @@ __device__ __forceinline__ void team_gather(const StageParams<T>& p, const T* so
   const Sched& sc = p.sc;
   const int lane = threadIdx.x & 31, el = lane % E, part = lane / E;
   const size_t ks = (size_t)sc.KS, fstride = (size_t)NP * ks, bstride = 3 * fstride;
-  const int e = tile * E + el;
+  // lanes past the last active element repeat it (and store nothing)
+  t.valid = tile < ntiles && tile * E + el < nactive;
+  const int e = t.valid ? tile * E + el : nactive - 1;
   t.e = e;
-  t.valid = tile < ntiles && e < nactive;
-  t.lev = 1;
-  t.a = 0;
-  t.rx = t.ry = t.sx = t.sy = T(0);
   T own[4][NB];
 #pragma unroll
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int n = 0; n < NB; ++n) own[f][n] = T(0);
   TeamFace<T, NFP> fc;
-  fc.nb = kWall;
-  fc.lower = false;
-  if (t.valid) {
-    if (part < 3) team_load_face<T, N>(p, e, part, k, fc);
+  if (tile < ntiles) {
+    const int4 cn = __ldg(p.s.conn + e);
+    t.finer = (cn.w >> 12) & 1;
+    if (part < 3) team_load_face<T, N>(p, cn, e, part, k, fc);
     t.lev = level_of(sc, e);
     t.a = k >> (t.lev - 1);
     const T* q = p.s.q + (size_t)(t.a & 1) * bstride + e;
@@ -384,7 +416,6 @@ __device__ __forceinline__ void team_gather(const StageParams<T>& p, const T* so
   T* sx = sw + C::FX + el * C::XS;
   if (part < 3) {
     const int f = part;
-    const bool in = fc.nb >= 0;
     const T Ef = fc.lower ? fc.E : E0, Bf = fc.lower ? fc.B : B0;
     T vx, vy;
     face_normal(f, t.rx, t.ry, t.sx, t.sy, vx, vy);
@@ -394,10 +425,10 @@ __device__ __forceinline__ void team_gather(const StageParams<T>& p, const T* so
 #pragma unroll
     for (int m = 0; m < NFP; ++m) {
       const T* o = so + face_node_rt(D::N, f, m);
-      tr[m][0] = pair(o[0] - Ef, in ? fc.v[0][m] - Ef : T(0));
-      tr[m][1] = pair(o[NPP], in ? fc.v[1][m] : T(0));
-      tr[m][2] = pair(o[2 * NPP], in ? fc.v[2][m] : T(0));
-      tr[m][3] = pair(o[3 * NPP] - Bf, in ? fc.v[3][m] - Bf : T(0));
+      tr[m][0] = add2(pair(o[0], fc.v[0][m]), dup(-Ef));
+      tr[m][1] = pair(o[NPP], fc.v[1][m]);
+      tr[m][2] = pair(o[2 * NPP], fc.v[2][m]);
+      tr[m][3] = add2(pair(o[3 * NPP], fc.v[3][m]), dup(-Bf));
     }
     if constexpr (C::FP64) {
       Pair<T>* sf = reinterpret_cast<Pair<T>*>(sw + C::FACE + el * C::FS) + f * NFP * 4;
@@ -411,7 +442,7 @@ __device__ __forceinline__ void team_gather(const StageParams<T>& p, const T* so
       sg[2] = nx;
       sg[3] = ny;
       sg[4] = hs;
-      sg[5] = in ? T(0) : T(fc.nb);   // kind: 0 interior, kWall, kFarField
+      sg[5] = fc.nb >= 0 ? T(0) : T(fc.nb);   // kind: 0 interior, kWall, kFarField
       sg[6] = vx;
       sg[7] = vy;
     } else {
@@ -488,7 +519,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   constexpr bool kRegs = sizeof(T) == 4;   // FP32 keeps the interpolated rows in registers
   const int lane = threadIdx.x & 31, el = lane % E, part = lane / E;
   const int i0 = L * NB == NPP || part < NPP ? part * NB : 0;   // a lane past NPP repeats node 0 (unused)
-  const T g = (T)p.ph.g, hvel = (T)p.ph.hvel;
+  const T g = phys_g(p.ph, T(0)), hvel = phys_hvel(p.ph, T(0));
   const T* so = sw + C::OWN + el * C::OS;
   const T h0 = E0 - B0;
   const T rx = t.rx, ry = t.ry, sx = t.sx, sy = t.sy;
@@ -574,7 +605,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
     const T am = mad(rx, huc, ry * hvc), bm = mad(sx, huc, sy * hvc);
     if constexpr (D::EXACT) {
       hc = h0 + hsum(a0);
-      const T ih = hc > hvel ? recip(hc) : T(0);
+      const T ih = hc > hvel ? recip_fast(hc) : T(0);
       const T u = huc * ih, v = hvc * ih, gm = -g * hc;
       F[0] = u * am; F[1] = v * am; F[2] = u * bm; F[3] = v * bm;
       F[4] = gm * mad(rx, dr, sx * ds);
@@ -582,7 +613,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
     } else {
       const T ec = hsum(a1), bc = hsum(a0);
       hc = h0 + (ec - bc);
-      const T ih = hc > hvel ? recip(hc) : T(0);
+      const T ih = hc > hvel ? recip_fast(hc) : T(0);
       const T u = huc * ih, v = hvc * ih, gm = -g * ec;
       const T pr = T(0.5) * g * ec * (ec - T(2) * bc);
       F[0] = mad(u, am, rx * pr); F[1] = mad(v, am, ry * pr); F[2] = mad(u, bm, sx * pr); F[3] = mad(v, bm, sy * pr);
@@ -745,6 +776,36 @@ __device__ __forceinline__ T team_min(T v) {
   return v;
 }
 
+// s[f] = sum over the lane's NB nodes of w q[f], f = eta, hu, hv (`on` false: zero).
+// Even NB: two nodes per packed instruction.
+template <typename T, int NB>
+__device__ __forceinline__ void node_sums(const T* w, bool on, const T (&q)[4][NB], T (&s)[3]) {
+  if constexpr (NB % 2 == 0) {
+    Pair<T> acc[3] = {dup(T(0)), dup(T(0)), dup(T(0))};
+#pragma unroll
+    for (int n = 0; n < NB; n += 2) {
+      const Pair<T> x = *reinterpret_cast<const Pair<T>*>(w + n);
+#pragma unroll
+      for (int f = 0; f < 3; ++f) acc[f] = fma2(x, pair(q[f][n], q[f][n + 1]), acc[f]);
+    }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) s[f] = on ? hsum(acc[f]) : T(0);
+  } else {
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      const T x = on ? w[n] : T(0);
+#pragma unroll
+      for (int f = 0; f < 3; ++f) s[f] = mad(x, q[f][n], s[f]);
+    }
+  }
+}
+
+// a mod 3 of a non-negative activation count: 2^32 = 1 (mod 3), so the halves add up and
+// one 32-bit remainder does
+__device__ __forceinline__ int ring_slot3(long long a) {
+  return (int)(((unsigned)a % 3u + (unsigned)((unsigned long long)a >> 32) % 3u) % 3u);
+}
+
 // Adams-Bashforth commit (Algorithm 1) and positivity limiter (Algorithm 3) of an
 // element whose nodes part * NB + n sit with lane (el, part) of a team of L lanes
 // (mode 0), or the R output in the caller's layout (mode 1). q: the state at the
@@ -753,8 +814,8 @@ __device__ __forceinline__ T team_min(T v) {
 // each field's increments are summed first and added to the state with the rounding
 // error of the previous update taken back.
 template <typename T, int N, int L, int NB, bool kComp>
-__device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* sops, bool valid, int e, int part,
-                                            int lev, long long a, T (&q)[4][NB], const T (&R)[3][NB], T rx, T ry,
+__device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* sops, bool valid, bool finer, int e,
+                                            int part, int lev, long long a, T (&q)[4][NB], const T (&R)[3][NB], T rx, T ry,
                                             T sx, T sy, double* injected) {
   using D = Dims<N>;
   using O = OpLayout<N>;
@@ -778,71 +839,55 @@ __device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* so
     const int depth = a + 1 < 3 ? (int)(a + 1) : 3;
     T wab[3], wh[3];
     ab_weights<T>(depth, wab);
+    ab_partial_weights<T>(depth, T(0.5), wh);
     const T dtl = level_dt(sc, lev, T(0));
     const T c0 = dtl * wab[0], c1 = dtl * wab[1], c2 = dtl * wab[2];
-    T* ring = p.s.ring + eo;
-    T* w0 = ring + (size_t)(a % 3) * bstride;
-    T r1[3][NB], r2[3][NB];
+    const T m0 = dtl * wh[0], m1 = dtl * wh[1], m2 = dtl * wh[2];
+    // finer: an element with a finer neighbour also stores the Adams-Bashforth polynomial
+    // of this step at its middle, q(t_a + dt/2) (Section 4), for that neighbour's next substep
+    const unsigned ks4 = (unsigned)sc.KS;
+    const size_t eb = eo + (size_t)((unsigned)i0 * ks4);   // the lane's first node in a field's planes
+    const int s0 = ring_slot3(a), s1 = s0 == 0 ? 2 : s0 - 1, s2 = s1 == 0 ? 2 : s1 - 1;
+    T* w0 = p.s.ring + (size_t)s0 * bstride + eb;
+    const T* p1 = p.s.ring + (size_t)s1 * bstride + eb;
+    const T* p2 = p.s.ring + (size_t)s2 * bstride + eb;
+    T* cp = kComp ? p.s.comp + eb : nullptr;
+    T* qm = p.s.qmid + eo * 3 * NPP + i0;
 #pragma unroll
-    for (int f = 0; f < 3; ++f)
+    for (int f = 0; f < 3; ++f) {   // one field's history at a time in registers
+      T r1[NB], r2[NB], ce[kComp ? NB : 1];
 #pragma unroll
-      for (int n = 0; n < NB; ++n) r1[f][n] = r2[f][n] = T(0);
-    if (depth > 1) {
-      const T* p1 = ring + (size_t)((a - 1) % 3) * bstride;
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-#pragma unroll
-        for (int n = 0; n < NB; ++n)
-          if (i0 + n < NP) r1[f][n] = ldm(p1 + f * fstride + (size_t)(i0 + n) * ks);
-    }
-    if (depth > 2) {
-      const T* p2 = ring + (size_t)((a - 2) % 3) * bstride;
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-#pragma unroll
-        for (int n = 0; n < NB; ++n)
-          if (i0 + n < NP) r2[f][n] = ldm(p2 + f * fstride + (size_t)(i0 + n) * ks);
-    }
-#pragma unroll
-    for (int f = 0; f < 3; ++f)
+      for (int n = 0; n < NB; ++n) {
+        const unsigned o = n * ks4;
+        const bool in = kAll && NB * (L - 1) + n < NP ? true : i0 + n < NP;
+        r1[n] = depth > 1 && in ? ldm(p1 + o) : T(0);
+        r2[n] = depth > 2 && in ? ldm(p2 + o) : T(0);
+        if constexpr (kComp) ce[n] = in ? ldm(cp + o) : T(0);
+      }
 #pragma unroll
       for (int n = 0; n < NB; ++n)
-        if (i0 + n < NP) w0[f * fstride + (size_t)(i0 + n) * ks] = R[f][n];
-    // The Adams-Bashforth polynomial of this step at its middle, q(t_a + dt/2)
-    // (Section 4), stored for a finer neighbour's next substep.
-    if ((__ldg(reinterpret_cast<const int*>(p.s.conn + e) + 3) >> 12) & 1) {
-      ab_partial_weights<T>(depth, T(0.5), wh);
-      const T m0 = dtl * wh[0], m1 = dtl * wh[1], m2 = dtl * wh[2];
-      T* qm = p.s.qmid + eo * 3 * NPP + i0;
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
+        if (kAll && NB * (L - 1) + n < NP ? true : i0 + n < NP) w0[n * ks4] = R[f][n];
+      if (finer) {
 #pragma unroll
         for (int n = 0; n < NB; ++n)
-          if (kAll || i0 + n < NPP) qm[f * NPP + n] = mad(m2, r2[f][n], mad(m1, r1[f][n], mad(m0, R[f][n], q[f][n])));
-    }
-    if constexpr (kComp) {
-      T* cp = p.s.comp + eo;
-      T ce[3][NB];
+          if (kAll || i0 + n < NPP)
+            qm[f * NPP + n] = mad(m2, r2[n], mad(m1, r1[n], mad(m0, R[f][n], q[f][n])));
+      }
 #pragma unroll
-      for (int f = 0; f < 3; ++f)
-#pragma unroll
-        for (int n = 0; n < NB; ++n)
-          ce[f][n] = i0 + n < NP ? ldm(cp + f * fstride + (size_t)(i0 + n) * ks) : T(0);
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-#pragma unroll
-        for (int n = 0; n < NB; ++n) {
-          // y = d - c, t = q + y, and the new error c = (t - q) - y
-          const T y = mad(c2, r2[f][n], mad(c1, r1[f][n], c0 * R[f][n])) - ce[f][n];
+      for (int n = 0; n < NB; ++n) {
+        if constexpr (kComp) {   // y = d - c, t = q + y, and the new error c = (t - q) - y
+          const T y = mad(c2, r2[n], mad(c1, r1[n], c0 * R[f][n])) - ce[n];
           const T s = q[f][n] + y;
-          if (i0 + n < NP) cp[f * fstride + (size_t)(i0 + n) * ks] = (s - q[f][n]) - y;
+          if (i0 + n < NP) cp[n * ks4] = (s - q[f][n]) - y;
           q[f][n] = s;
+        } else {
+          q[f][n] = mad(c2, r2[n], mad(c1, r1[n], mad(c0, R[f][n], q[f][n])));
         }
-    } else {
-#pragma unroll
-      for (int f = 0; f < 3; ++f)
-#pragma unroll
-        for (int n = 0; n < NB; ++n) q[f][n] = mad(c2, r2[f][n], mad(c1, r1[f][n], mad(c0, R[f][n], q[f][n])));
+      }
+      w0 += fstride;
+      p1 += fstride;
+      p2 += fstride;
+      if constexpr (kComp) cp += fstride;
     }
   }
 
@@ -866,12 +911,7 @@ __device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* so
   int dryf = 0;
   {
     T s[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-      const T w = kAll || i0 < NPP ? sops[O::MW + ir + n] : T(0);   // zero in the padding
-#pragma unroll
-      for (int f = 0; f < 3; ++f) s[f] = mad(w, q[f][n], s[f]);
-    }
+    node_sums<T, NB>(sops + O::MW + ir, kAll || i0 < NPP, q, s);   // zero weights in the padding
 #pragma unroll
     for (int f = 0; f < 3; ++f) me[f] = team_sum<L>(s[f]);
   }
@@ -950,22 +990,19 @@ __device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* so
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     T s[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-      const T w = kAll || i0 < NPP ? sops[O::T1 + k * NPP + ir + n] : T(0);
-#pragma unroll
-      for (int f = 0; f < 3; ++f) s[f] = mad(w, q[f][n], s[f]);
-    }
+    node_sums<T, NB>(sops + O::T1 + k * NPP + ir, kAll || i0 < NPP, q, s);
 #pragma unroll
     for (int f = 0; f < 3; ++f) v1[f][k] = team_sum<L>(s[f]);
   }
   if (!valid) return;
-  T* qd = p.s.q + (size_t)((a + 1) & 1) * bstride + eo;
+  T* qd = p.s.q + (size_t)((a + 1) & 1) * bstride + eo + (size_t)((unsigned)i0 * (unsigned)sc.KS);
 #pragma unroll
-  for (int f = 0; f < 3; ++f)
+  for (int f = 0; f < 3; ++f) {
 #pragma unroll
     for (int n = 0; n < NB; ++n)
-      if (i0 + n < NP) qd[f * fstride + (size_t)(i0 + n) * ks] = q[f][n];
+      if (kAll && NB * (L - 1) + n < NP ? true : i0 + n < NP) qd[n * (unsigned)sc.KS] = q[f][n];
+    qd += fstride;
+  }
   // the element's small records, dealt to the lanes of the team: lane f < 3 (with two
   // lanes, lane 0 also field 1) stores field f
 #pragma unroll
@@ -996,7 +1033,7 @@ __device__ __forceinline__ void team_compute(const StageParams<T>& p, const T* s
   for (int f = 0; f < 4; ++f)
 #pragma unroll
     for (int n = 0; n < NB; ++n) q[f][n] = so[f * NPP + ir + n];
-  team_commit<T, N, C::L, NB, kComp>(p, sops, t.valid, t.e, part, t.lev, t.a, q, R, t.rx, t.ry, t.sx, t.sy, injected);
+  team_commit<T, N, C::L, NB, kComp>(p, sops, t.valid, t.finer, t.e, part, t.lev, t.a, q, R, t.rx, t.ry, t.sx, t.sy, injected);
   __syncwarp();   // the tile's rows are read before the next gather overwrites them
 }
 

@@ -274,6 +274,11 @@ swe::Phys phys_of(const swe_solver* s, int mask) {
   ph.ff_h = s->ff[0];
   ph.ff_hu = s->ff[1];
   ph.ff_hv = s->ff[2];
+  ph.g_f = (float)ph.g;
+  ph.hvel_f = (float)ph.hvel;
+  ph.ff_h_f = (float)ph.ff_h;
+  ph.ff_hu_f = (float)ph.ff_hu;
+  ph.ff_hv_f = (float)ph.ff_hv;
   return ph;
 }
 
@@ -391,84 +396,72 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
   put_rows(O::PST, e.Ps, nc, np, true);
   put_rows(O::PT, e.P, nc, np, true);
 
-  {
-  // tensor-core fragments (mma.sync m16n8k16 / m16n8k8 bf16 B operands)
+  // tensor-core fragments (mma.sync m16n8k16 / m16n8k8 bf16 B operands): lane (g, t)
+  // holds column n = g, rows k = 2t, 2t+1 (and 2t+8, 2t+9)
   tc.assign(TL::SIZE, 0u);
   const std::vector<double>* interp[3] = {&e.Ic, &e.Icr, &e.Ics};   // nc x np
   const std::vector<double>* proj[3] = {&e.Pr, &e.Ps, &e.P};        // np x nc
   auto pack2 = [](uint16_t lo16, uint16_t hi16) { return (uint32_t)lo16 | ((uint32_t)hi16 << 16); };
-  for (int op = 0; op < 3; ++op)
+  // a k16 fragment (hi 2, lo 2 words) of B[k][n] at words d
+  auto put16 = [&](size_t d, int lane, auto&& Bv) {
+    const int g = lane / 4, t = lane % 4;
+    const int kk[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
+    uint16_t h[4], l[4];
+    for (int q = 0; q < 4; ++q) bf16_split(Bv(kk[q], g), h[q], l[q]);
+    tc[d + 0] = pack2(h[0], h[1]);
+    tc[d + 1] = pack2(h[2], h[3]);
+    tc[d + 2] = pack2(l[0], l[1]);
+    tc[d + 3] = pack2(l[2], l[3]);
+  };
+  // a k8 fragment (hi, lo)
+  auto put8 = [&](size_t d, int lane, auto&& Bv) {
+    const int g = lane / 4, t = lane % 4;
+    uint16_t h0, l0, h1, l1;
+    bf16_split(Bv(2 * t, g), h0, l0);
+    bf16_split(Bv(2 * t + 1, g), h1, l1);
+    tc[d + 0] = pack2(h0, h1);
+    tc[d + 1] = pack2(l0, l1);
+  };
+  for (int lane = 0; lane < 32; ++lane) {
     for (int ct = 0; ct < C::CT; ++ct)
-      for (int ks = 0; ks < C::KSTEP; ++ks)
-        for (int lane = 0; lane < 32; ++lane) {
-          const int g = lane / 4, t = lane % 4;
-          // B[k][n] = Op[c = 8ct + n][j = 16ks + k]
-          auto Bv = [&](int kk, int nn) {
-            const int c = 8 * ct + nn, j = 16 * ks + kk;
+      for (int op = 0; op < 3; ++op) {
+        for (int ks = 0; ks < C::KSTEP; ++ks)
+          put16(TL::INTERP + ((((size_t)ct * 3 + op) * C::KSTEP + ks) * 32 + lane) * 4, lane, [&](int kk, int nn) {
+            const int c = 8 * ct + nn, j = 16 * ks + kk;   // B[k][n] = Op[c][j]
             return (c < nc && j < np) ? (*interp[op])[(size_t)c * np + j] : 0.0;
-          };
-          const int kk[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
-          uint16_t h[4], l[4];
-          for (int q = 0; q < 4; ++q) bf16_split(Bv(kk[q], g), h[q], l[q]);
-          const size_t base = (((size_t)(op * C::CT + ct) * C::KSTEP + ks) * 2) * 64;
-          tc[TL::INTERP + base + 0 * 64 + lane * 2 + 0] = pack2(h[0], h[1]);
-          tc[TL::INTERP + base + 0 * 64 + lane * 2 + 1] = pack2(h[2], h[3]);
-          tc[TL::INTERP + base + 1 * 64 + lane * 2 + 0] = pack2(l[0], l[1]);
-          tc[TL::INTERP + base + 1 * 64 + lane * 2 + 1] = pack2(l[2], l[3]);
-        }
-  for (int op = 0; op < 3; ++op)
-    for (int ct = 0; ct < C::CT; ++ct)
-      for (int nt = 0; nt < C::NT; ++nt)
-        for (int lane = 0; lane < 32; ++lane) {
-          const int g = lane / 4, t = lane % 4;
-          // B[k][n] = Op[i = 8nt + n][c = 8ct + k]
-          auto Bv = [&](int kk, int nn) {
-            const int i = 8 * nt + nn, c = 8 * ct + kk;
+          });
+        for (int nt = 0; nt < C::NT; ++nt)
+          put8(TL::PROJ + ((((size_t)ct * C::NT + nt) * 3 + op) * 32 + lane) * 2, lane, [&](int kk, int nn) {
+            const int i = 8 * nt + nn, c = 8 * ct + kk;    // B[k][n] = Op[i][c]
             return (i < np && c < nc) ? (*proj[op])[(size_t)i * nc + c] : 0.0;
-          };
-          uint16_t h0, l0, h1, l1;
-          bf16_split(Bv(2 * t, g), h0, l0);
-          bf16_split(Bv(2 * t + 1, g), h1, l1);
-          const size_t base = (((size_t)(op * C::CT + ct) * C::NT + nt) * 2) * 32;
-          tc[TL::PROJ + base + 0 * 32 + lane] = pack2(h0, h1);
-          tc[TL::PROJ + base + 1 * 32 + lane] = pack2(l0, l1);
-        }
-  // nodal differentiation for the strong-form pressure term: TF32 m16n8k8 B
-  // operands, B[k][n] = D[i = 8nt + n][j = 8kk + k]; lane (g, t) holds k = t, t + 4
-  for (int op = 0; op < 2; ++op)
-    for (int kk = 0; kk < C::KP / 8; ++kk)
-      for (int nt = 0; nt < C::NT; ++nt)
-        for (int lane = 0; lane < 32; ++lane) {
+          });
+      }
+    for (int nt = 0; nt < C::NT; ++nt) {
+      for (int op = 0; op < 2; ++op) {
+        for (int ks = 0; ks < C::KSTEP; ++ks)
+          put16(TL::MASS + ((((size_t)op * C::KSTEP + ks) * C::NT + nt) * 32 + lane) * 4, lane, [&](int kk, int nn) {
+            const int i = 8 * nt + nn, j = 16 * ks + kk;
+            return (i < np && j < np) ? o[(op == 0 ? O::WR : O::WS) + (size_t)i * npp + j] : 0.0;
+          });
+        // nodal differentiation for the strong-form pressure term, TF32 m16n8k8: lane
+        // (g, t) holds column n = g, rows k = t, t + 4
+        for (int kk = 0; kk < C::KP / 8; ++kk) {
           const int g = lane / 4, t = lane % 4;
           auto Bv = [&](int k, int n) {
             const int i = 8 * nt + n, j = 8 * kk + k;
             return (i < np && j < np) ? o[(op == 0 ? O::DR : O::DS) + (size_t)i * npp + j] : 0.0;
           };
-          uint32_t h0, l0, h1, l1;
-          tf32_split(Bv(t, g), h0, l0);
-          tf32_split(Bv(t + 4, g), h1, l1);
-          const size_t base = TL::DIFF + ((((size_t)op * (C::KP / 8) + kk) * C::NT + nt) * 2) * 64;
-          tc[base + 0 * 64 + lane * 2 + 0] = h0;
-          tc[base + 0 * 64 + lane * 2 + 1] = h1;
-          tc[base + 1 * 64 + lane * 2 + 0] = l0;
-          tc[base + 1 * 64 + lane * 2 + 1] = l1;
+          const size_t d = TL::DIFF + ((((size_t)op * (C::KP / 8) + kk) * C::NT + nt) * 32 + lane) * 4;
+          tf32_split(Bv(t, g), tc[d + 0], tc[d + 2]);
+          tf32_split(Bv(t + 4, g), tc[d + 1], tc[d + 3]);
         }
-  // lift: B[k][n] = -Lg[i = 8nt + n][q = 8kt + k], q = 3 Ng face points (Lg is np x 3ng)
-  for (int kt = 0; kt < C::KT; ++kt)
-    for (int nt = 0; nt < C::NT; ++nt)
-      for (int lane = 0; lane < 32; ++lane) {
-        const int g = lane / 4, t = lane % 4;
-        auto Bv = [&](int kk, int nn) {
+      }
+      for (int kt = 0; kt < C::KT; ++kt)   // lift: B[k][n] = -Lg[i][q], q = 3 Ng face points (Lg is np x 3ng)
+        put8(TL::LIFT + (((size_t)kt * C::NT + nt) * 32 + lane) * 2, lane, [&](int kk, int nn) {
           const int i = 8 * nt + nn, q = 8 * kt + kk;
           return (i < np && q < 3 * ng) ? -e.Lg[(size_t)i * 3 * ng + q] : 0.0;
-        };
-        uint16_t h0, l0, h1, l1;
-        bf16_split(Bv(2 * t, g), h0, l0);
-        bf16_split(Bv(2 * t + 1, g), h1, l1);
-        const size_t base = ((size_t)(kt * C::NT + nt) * 2) * 32;
-        tc[TL::LIFT + base + 0 * 32 + lane] = pack2(h0, h1);
-        tc[TL::LIFT + base + 1 * 32 + lane] = pack2(l0, l1);
-      }
+        });
+    }
   }
 }
 
@@ -606,6 +599,7 @@ int upload_mesh_t(swe_solver* s) {
       const int fn = nb >= 0 ? m.EToF[3 * (size_t)c + f] : 0;
       w |= (fn & 3) << (2 * f);
       w |= (jsel[3 * (size_t)c + f] & 3) << (6 + 2 * f);
+      w |= (s->level[nb >= 0 ? nb : c] - 1) << (13 + 3 * f);
       tvbg[8 * (size_t)e + 2 * f] = (T)alpha[3 * (size_t)c + f];
       tvbg[8 * (size_t)e + 2 * f + 1] = (T)beta[3 * (size_t)c + f];
     }
@@ -1728,6 +1722,7 @@ int swe_set_launch_config(swe_solver* s, int32_t ctas_per_sm) {
 int swe_set_tc_warps(swe_solver* s, int32_t warps) {
   if (!s) return fail(SWE_EINVAL, "bad arguments");
   if (!s->tc) return fail(SWE_EUNSUPPORTED, "warps per CTA apply to the FP32 tensor-core tier only");
+  if (warps > 8) return fail(SWE_EINVAL, "that many warps per CTA do not fit on an SM (1..8)");
   swe::KernelCfg c = s->cfg_max;
   const cudaError_t e = s->lf->tc_config(&c, warps);
   if (e == cudaErrorInvalidValue) return fail(SWE_EINVAL, "that many warps per CTA do not fit on an SM (1..8)");
