@@ -174,6 +174,7 @@ struct StageParams : ScnParams<T> {
   int j;          // substep within the macro step
   int nactive;    // elements [0, nactive) are active
   int mode;       // 0: R + commit + positivity; 1: R only, written to out
+  int early;      // the next kernel's CTAs may start while this one runs (else when its warps are done)
   T* out;         // mode 1: [3][K][NP], caller order
   const int* perm;
 };
@@ -183,6 +184,7 @@ struct LimitParams : ScnParams<T> {
   int j;
   int nactive;
   int post_stage;  // 1: limit the just-committed state of active elements; 0: current state
+  int early;       // as StageParams::early
 };
 
 // ---- persistent batched launch ------------------------------------------

@@ -132,9 +132,42 @@ __device__ __forceinline__ double sqrt_nn(double x) { return sqrt(x); }
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
 
+// a b + c in one rounding. Every product that meets a sum in the stage and limiter bodies
+// is written with it (or with fma2): left to the compiler, a b + c d is fused on either
+// side, and the separate launch and the batch kernel would round differently.
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+// Hardware reciprocal and inverse square root without the scaling that the plain calls
+// spend on subnormal arguments (three more instructions each): depths above the dry
+// threshold and squared speeds are normal numbers. FP64: the correctly rounded ones.
+__device__ __forceinline__ float recip_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double recip_fast(double x) { return 1.0 / x; }
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt_t(x); }
+// |u| + sqrt(x), x >= 0 (FP32: the square root as in sqrt_nn)
+__device__ __forceinline__ float speed(float u, float x) { return mad(x, rsqrt_fast(fmaxf(x, 1e-30f)), fabsf(u)); }
+__device__ __forceinline__ double speed(double u, double x) { return fabs(u) + sqrt(x); }
+
+
 // Cache hints: start a line's trip from memory early, without holding registers.
 // Only addresses inside live buffers are ever passed.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// Programmatic dependent launch. The kernels of a substep run one after the other on one
+// stream; each lets the next one's CTAs start (dependents_may_launch), at its own start or
+// when its warps are done with their elements (`early`), and itself reads only what no
+// kernel writes (operators) before wait_for_previous, which returns when the kernel before
+// it has completed and its stores are visible. Every kernel launched with launch_dependent (launch.hpp) calls it.
+__device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Loads of the arrays the kernels write (state, Adams-Bashforth history, half-step
 // records, means, dry flags, P1 values): ordinary coherent global loads, never the
@@ -179,6 +212,18 @@ __device__ __forceinline__ float level_dt(const Sched& sc, int l, float) { retur
 __device__ __forceinline__ double level_dt(const Sched& sc, int l, double) { return sc.dtl_d[l - 1]; }
 __device__ __forceinline__ float eps_of(const Phys& ph, float) { return ph.eps_f; }
 __device__ __forceinline__ double eps_of(const Phys& ph, double) { return ph.eps; }
+
+__device__ __forceinline__ float phys_g(const Phys& ph, float) { return ph.g_f; }
+__device__ __forceinline__ double phys_g(const Phys& ph, double) { return ph.g; }
+__device__ __forceinline__ float phys_hvel(const Phys& ph, float) { return ph.hvel_f; }
+__device__ __forceinline__ double phys_hvel(const Phys& ph, double) { return ph.hvel; }
+__device__ __forceinline__ float phys_ff(const Phys& ph, int c, float) {
+  return c == 0 ? ph.ff_h_f : (c == 1 ? ph.ff_hu_f : ph.ff_hv_f);
+}
+__device__ __forceinline__ double phys_ff(const Phys& ph, int c, double) {
+  return c == 0 ? ph.ff_h : (c == 1 ? ph.ff_hu : ph.ff_hv);
+}
+
 
 __host__ __device__ constexpr int face_node(int N, int f, int m) {
   // node index of position m along face f (from vertex f to f+1), lattice order
@@ -700,10 +745,13 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 3) k_tvb(const __grid_constant__ LimitParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sops = reinterpret_cast<T*>(smem_raw);
+  if (p.early) dependents_may_launch();
   stage_ops<T, N, OpLayout<N>::TAIL>(sops, p.s.ops);
+  wait_for_previous();
   const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
   tvb_range<T, N>(p, p.post_stage, sops, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nactive,
                   k);
+  if (!p.early) dependents_may_launch();
 }
 
 }  // namespace swe

@@ -73,7 +73,11 @@ const Launchers<double>* launchers_for<double>(int N) {
 
 namespace {
 
-__global__ void k_advance(long long* macro) { *macro += 1; }
+__global__ void k_advance(long long* macro) {
+  dependents_may_launch();
+  wait_for_previous();
+  *macro += 1;
+}
 
 __global__ void k_stats_finalize(const double* partials, int nblocks, double* out) {
   __shared__ double sm[256];
@@ -367,8 +371,7 @@ template cudaError_t launch_unpack_state<double>(const double*, const double*, c
                                                  int, double*, cudaStream_t);
 
 cudaError_t launch_advance(long long* macro, cudaStream_t st) {
-  k_advance<<<1, 1, 0, st>>>(macro);
-  return cudaGetLastError();
+  return launch_dependent(k_advance, 1, 1, 0, st, macro);
 }
 
 cudaError_t launch_stats_finalize(const double* partials, int nblocks, double* out, cudaStream_t st) {

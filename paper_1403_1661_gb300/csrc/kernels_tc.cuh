@@ -619,14 +619,17 @@ __global__ void __launch_bounds__(32 * TcSmem<N>::LIMIT, 1) k_stage_tc(const __g
   using SM = TcSmem<N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sops = reinterpret_cast<float*>(smem_raw);
+  if (p.early) dependents_may_launch();
   tc_ops_begin<N>(sops, p.s.ops, p.s.tcops);
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   float* sw = sops + SM::CTA + warp * SM::WARP;
   stage_tc_init<N>(sw);
+  wait_for_previous();
   const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
   const int ntiles = (p.nactive + SM::E - 1) / SM::E;
   const double injected =
       stage_tc_range<N, kComp>(p, k, p.nactive, sops, sw, blockIdx.x * nw + warp, gridDim.x * nw, ntiles, true, true);
+  if (!p.early) dependents_may_launch();
   if (injected != 0.0) atomicAdd(p.s.acc, injected);
 }
 

@@ -78,41 +78,6 @@ __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
 __device__ __forceinline__ double2 dup(double x) { return make_double2(x, x); }
 template <typename P>
 __device__ __forceinline__ auto hsum(P a) { return a.x + a.y; }
-// a b + c in one rounding. Every product that meets a sum in this file is written with
-// it (or with fma2): left to the compiler, a b + c d is fused on either side, and the
-// separate launch and the batch kernel would round differently.
-__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
-// Hardware reciprocal and inverse square root without the scaling that the plain calls
-// spend on subnormal arguments (three more instructions each): depths above the dry
-// threshold and squared speeds are normal numbers. FP64: the correctly rounded ones.
-__device__ __forceinline__ float recip_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ double recip_fast(double x) { return 1.0 / x; }
-__device__ __forceinline__ float rsqrt_fast(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt_t(x); }
-// |u| + sqrt(x), x >= 0 (FP32: the square root as in sqrt_nn)
-__device__ __forceinline__ float speed(float u, float x) { return mad(x, rsqrt_fast(fmaxf(x, 1e-30f)), fabsf(u)); }
-__device__ __forceinline__ double speed(double u, double x) { return fabs(u) + sqrt(x); }
-
-__device__ __forceinline__ float phys_g(const Phys& ph, float) { return ph.g_f; }
-__device__ __forceinline__ double phys_g(const Phys& ph, double) { return ph.g; }
-__device__ __forceinline__ float phys_hvel(const Phys& ph, float) { return ph.hvel_f; }
-__device__ __forceinline__ double phys_hvel(const Phys& ph, double) { return ph.hvel; }
-__device__ __forceinline__ float phys_ff(const Phys& ph, int c, float) {
-  return c == 0 ? ph.ff_h_f : (c == 1 ? ph.ff_hu_f : ph.ff_hv_f);
-}
-__device__ __forceinline__ double phys_ff(const Phys& ph, int c, double) {
-  return c == 0 ? ph.ff_h : (c == 1 ? ph.ff_hu : ph.ff_hv);
-}
-
 // four consecutive values (16-byte aligned) as two pairs
 __device__ __forceinline__ void load4(const float* p, float2 (&o)[2]) {
   const float4 v = *reinterpret_cast<const float4*>(p);
@@ -1061,6 +1026,7 @@ __global__ void __launch_bounds__(32 * Team<T, N>::MAXW, Team<T, N>::MINB)
   using C = Team<T, N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* smem = reinterpret_cast<T*>(smem_raw);
+  if (p.early) dependents_may_launch();
   const T *sops = smem, *spj = smem + C::PRE;
   T* sw = smem + (threadIdx.x >> 5) * C::WARP;
   if constexpr (kGlobalOps) {
@@ -1070,6 +1036,7 @@ __global__ void __launch_bounds__(32 * Team<T, N>::MAXW, Team<T, N>::MINB)
     sw += C::OPS;
     team_ops_begin<T, N>(smem, p.s.ops);
   }
+  wait_for_previous();
   const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
   const int ntiles = (p.nactive + C::E - 1) / C::E;
   const int nw = blockDim.x >> 5, step = gridDim.x * nw;
@@ -1083,6 +1050,7 @@ __global__ void __launch_bounds__(32 * Team<T, N>::MAXW, Team<T, N>::MINB)
     team_compute<T, N, kComp>(p, sops, spj, sw, t, &injected);
     tile += step;
   }
+  if (!p.early) dependents_may_launch();
   if (injected != 0.0) atomicAdd(p.s.acc, injected);
 }
 

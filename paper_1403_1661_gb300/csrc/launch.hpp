@@ -47,7 +47,35 @@ struct Launchers {
   // shared memory and grids in cfg; cudaErrorInvalidValue when that many warps'
   // tiles do not fit on an SM.
   cudaError_t (*tc_config)(KernelCfg* cfg, int warps);
+  // Whether the CTAs of a kernel over n elements may be placed while the one before it
+  // still runs (kind 0: stage kernel, tc: its tensor-core form; 1: TVB limiter): they go to
+  // the SMs that have room first, several to an SM. With at most one warp per SM that is
+  // harmless and takes the start-up off the step (2,048 elements, N = 2: 95 against 105 us
+  // per macro step); a grid of a few warps per SM ends up on part of the SMs (45 k
+  // elements, N = 3: 223 against 209 us), and one that fills the GPU gains nothing (500 k,
+  // N = 4: 1.294 against 1.285 ms). FP64 kernels, bound by the FP64 pipe of each SM, wait.
+  bool (*early)(int kind, bool tc, int n, const KernelCfg&);
 };
+
+// Launch a kernel that may start while the stream's previous kernel drains (programmatic
+// dependent launch; the kernel itself waits for that one before it reads what it wrote).
+// A launch otherwise costs its latency and the previous kernel's tail: about 2 us of each
+// of the 17 kernels of a 4-level macro step.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t st,
+                             const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // Registered per order by kernels_n*.cu; nullptr when the order is not built.
 template <typename T>

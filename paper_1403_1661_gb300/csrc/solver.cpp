@@ -692,6 +692,7 @@ int launch_limit_t(swe_solver* s, int mask, int post_stage, int j, int nactive) 
   p.j = j;
   p.nactive = nactive;
   p.post_stage = post_stage;
+  p.early = 0;
   if ((mask & SWE_LIM_PP) && !post_stage) {
     SWE_CUDA(lt->positivity(p, s->cfg, s->stream));
     s->launches++;
@@ -756,6 +757,12 @@ int enqueue_substep_t(swe_solver* s, int j, KernelTimer* tm = nullptr) {
   p.mode = 0;
   p.out = nullptr;
   p.perm = nullptr;
+  // the kernel after the stage is the TVB limiter of the same elements, or (without it)
+  // the next substep's stage; after the last substep comes the counter's update
+  const int period = 1 << (s->L - 1);
+  const bool last = j == period - 1, tvb = (s->prm.limiter_mask & SWE_LIM_TVB) != 0;
+  const bool next_stage = !last && lt->early(0, s->tc, s->off[active_levels(s, j + 1)], s->cfg);
+  p.early = tvb ? lt->early(1, s->tc, nactive, s->cfg) : next_stage;
   int rc;
   if ((rc = timer_mark(s, tm, true, 0, nactive))) return rc;
   if (s->tc) {
@@ -773,13 +780,13 @@ int enqueue_substep_t(swe_solver* s, int j, KernelTimer* tm = nullptr) {
     lp.j = j;
     lp.nactive = nactive;
     lp.post_stage = 1;
+    lp.early = next_stage;
     if ((rc = timer_mark(s, tm, true, 1, nactive))) return rc;
     SWE_CUDA(lt->tvb(lp, s->cfg, s->stream));
     if ((rc = timer_mark(s, tm, false, 1, 0))) return rc;
     ++nl;
   }
-  const int period = 1 << (s->L - 1);
-  if (j == period - 1) {
+  if (last) {
     if ((rc = timer_mark(s, tm, true, 2, 0))) return rc;
     SWE_CUDA(swe::launch_advance(p.s.macro, s->stream));
     if ((rc = timer_mark(s, tm, false, 2, 0))) return rc;
@@ -1388,6 +1395,7 @@ int swe_rhs(swe_solver* s, void* dev_R) {
     p.j = 0;
     p.nactive = s->K;
     p.mode = 1;
+    p.early = 0;
     p.out = reinterpret_cast<double*>(dev_R);
     p.perm = reinterpret_cast<const int*>(s->ws + s->lay.perm);
     SWE_CUDA(s->ld->stage(p, s->cfg, s->stream));
@@ -1399,6 +1407,7 @@ int swe_rhs(swe_solver* s, void* dev_R) {
     p.j = 0;
     p.nactive = s->K;
     p.mode = 1;
+    p.early = 0;
     p.out = reinterpret_cast<float*>(dev_R);
     p.perm = reinterpret_cast<const int*>(s->ws + s->lay.perm);
     if (s->tc) {
@@ -1435,6 +1444,7 @@ int rhs_variant_t(swe_solver* s, const swe::Launchers<T>* lt, int variant, T* R,
   p.j = 0;
   p.nactive = s->K;
   p.mode = 1;
+  p.early = 0;
   p.out = R;
   p.perm = reinterpret_cast<const int*>(s->ws + s->lay.perm);
   if (variant == SWE_RHS_FUSED) {
