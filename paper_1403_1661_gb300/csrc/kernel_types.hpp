@@ -157,7 +157,7 @@ struct Phys {
   int pp, dry_mode;
   // single-precision copies: a conversion in the kernel runs on the FP64 pipe (two lanes
   // per SM and clock) and holds its warp for 64 clocks
-  float g_f, hvel_f, ff_h_f, ff_hu_f, ff_hv_f;
+  float g_f, hvel_f, h0_f, tvb_M_f, tvb_nu_f, ff_h_f, ff_hu_f, ff_hv_f;
 };
 
 // One scenario: its device arrays, schedule and physics. The limiter bodies read

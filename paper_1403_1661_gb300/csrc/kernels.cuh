@@ -224,6 +224,12 @@ __device__ __forceinline__ double phys_ff(const Phys& ph, int c, double) {
   return c == 0 ? ph.ff_h : (c == 1 ? ph.ff_hu : ph.ff_hv);
 }
 
+__device__ __forceinline__ float phys_h0(const Phys& ph, float) { return ph.h0_f; }
+__device__ __forceinline__ double phys_h0(const Phys& ph, double) { return ph.h0; }
+__device__ __forceinline__ float phys_M(const Phys& ph, float) { return ph.tvb_M_f; }
+__device__ __forceinline__ double phys_M(const Phys& ph, double) { return ph.tvb_M; }
+__device__ __forceinline__ float phys_nu(const Phys& ph, float) { return ph.tvb_nu_f; }
+__device__ __forceinline__ double phys_nu(const Phys& ph, double) { return ph.tvb_nu; }
 
 __host__ __device__ constexpr int face_node(int N, int f, int m) {
   // node index of position m along face f (from vertex f to f+1), lattice order
@@ -532,224 +538,198 @@ __device__ __forceinline__ T minmod_tvb(T a, T b, T thr, bool& changed) {
   return r;
 }
 
+__device__ __forceinline__ float sqrt_fast(float x) { return x * rsqrt_fast(x); }
+__device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
+
 // The TVB limiter with the positivity modification on element e (k: the finest
 // substep count of the schedule); returns without change for an element that is dry,
-// has a dry neighbour or needs no limiting.
+// has a dry neighbour or needs no limiting. ops: the operator block (shared or global
+// memory; only an element that is limited reads it).
+//
+// What bounds it: the latency of its two dependent trips to memory (connectivity, then
+// the neighbours' means) and of the arithmetic between them; small launches hardly fill
+// a warp per scheduler. So the characteristic variables use the eigenvectors' closed-form
+// inverse (one reciprocal per element instead of a 3 x 3 inverse per edge), the kernel
+// stages nothing in shared memory, and the body is inlined with its parameters in the
+// constant bank (as an out-of-line function it read them through generic loads).
 template <typename T, int N>
-__device__ __forceinline__ void tvb_element(const ScnParams<T>& p, int post_stage, const T* __restrict__ sops,
-                                            int e, long long k) {
+__device__ __forceinline__ void tvb_element(const ScnParams<T>& p, int post_stage, const T* ops, int e, long long k) {
   using D = Dims<N>;
   using O = OpLayout<N>;
-  constexpr int NP = D::NP, NPP = D::NPP;
+  constexpr int NP = D::NP;
   const Sched& sc = p.sc;
-  const T g = (T)p.ph.g, h0 = (T)p.ph.h0;
-  {
-    // Every load is issued before the first branch on loaded data (an element that is
-    // dry or has a dry neighbour is skipped afterwards), so the latencies overlap:
-    // two dependent trips to memory (connectivity, then the neighbours) instead of four.
-    const int4 cn = __ldg(p.s.conn + e);
-    const int de = ldm(p.s.dry + e);
-    const int nbs[3] = {cn.x, cn.y, cn.z};
-    const int lev = level_of(sc, e);
-    const long long a = k >> (lev - 1);
-    const int cur = (int)((a + post_stage) & 1);
-    const size_t ks = (size_t)sc.KS, fstride = (size_t)NP * ks, bstride = 3 * fstride, eo = (size_t)e;
-    T* q = p.s.q + cur * bstride;
-    // 16-byte rows: geometry, element means (eta, hu, hv, -) as stored by the
-    // positivity pass, the neighbour-mean weights
-    T gm[4], u0[4], tg[8];
-    load_row_global<T, 4>(p.s.geo + 4 * eo, gm);
-    load_row_m<T, 4>(p.s.means + 4 * eo, u0);
-    load_row_global<T, 8>(p.s.tvbg + 8 * eo, tg);
-    // P1 part: vertex values of Pi1 q for eta, hu, hv (stored with the committed
-    // state) and of Pi1 B (static)
-    T vq[3][3], vb[3];
+  const T g = phys_g(p.ph, T(0)), h0 = phys_h0(p.ph, T(0));
+  // Every load is issued before the first branch on loaded data (an element that is
+  // dry or has a dry neighbour is skipped afterwards), so the latencies overlap.
+  const int4 cn = __ldg(p.s.conn + e);
+  const int de = ldm(p.s.dry + e);
+  const int nbs[3] = {cn.x, cn.y, cn.z};
+  const int lev = level_of(sc, e);
+  const long long a = k >> (lev - 1);
+  const int cur = (int)((a + post_stage) & 1);
+  const size_t ks = (size_t)sc.KS, fstride = (size_t)NP * ks, bstride = 3 * fstride, eo = (size_t)e;
+  T* q = p.s.q + cur * bstride + eo;
+  // 16-byte rows: geometry, element means (eta, hu, hv, -) as stored by the
+  // positivity pass, the neighbour-mean weights
+  T gm[4], u0[4], tg[8];
+  load_row_global<T, 4>(p.s.geo + 4 * eo, gm);
+  load_row_m<T, 4>(p.s.means + 4 * eo, u0);
+  load_row_global<T, 8>(p.s.tvbg + 8 * eo, tg);
+  // P1 part: vertex values of Pi1 q for eta, hu, hv (stored with the committed state)
+  T vq[3][3];
 #pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      vq[0][v] = ldm(p.s.p1 + (0 + v) * ks + eo);
-      vq[1][v] = ldm(p.s.p1 + (3 + v) * ks + eo);
-      vq[2][v] = ldm(p.s.p1 + (6 + v) * ks + eo);
-      vb[v] = __ldg(p.s.vb + v * ks + eo);
+  for (int v = 0; v < 3; ++v) {
+    vq[0][v] = ldm(p.s.p1 + (0 + v) * ks + eo);
+    vq[1][v] = ldm(p.s.p1 + (3 + v) * ks + eo);
+    vq[2][v] = ldm(p.s.p1 + (6 + v) * ks + eo);
+  }
+  const double Bbar_d = __ldg(p.s.Bbar + eo);
+  // neighbour means and dry flags
+  T un[3][4];
+  int dn = 0;
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const int nb = nbs[f] < 0 ? e : nbs[f];   // a boundary face reads its own element's (replaced below)
+    dn |= nbs[f] < 0 ? 0 : (int)ldm(p.s.dry + nb);
+    load_row_m<T, 4>(p.s.means + 4 * (size_t)nb, un[f]);
+  }
+  if (de || dn) return;
+  const T rx = gm[0], ry = gm[1], sx = gm[2], sy = gm[3];
+  const T Bbar = (T)Bbar_d;
+  // a far-field face sees the far-field state over the own mean bed; a wall face
+  // mirrors the normal momentum of the own mean
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    if (nbs[f] >= 0) continue;
+    if (nbs[f] == kFarField) {
+      un[f][0] = phys_ff(p.ph, 0, T(0)) + Bbar;
+      un[f][1] = phys_ff(p.ph, 1, T(0));
+      un[f][2] = phys_ff(p.ph, 2, T(0));
+    } else {
+      const T vxn = f == 0 ? -sx : (f == 1 ? rx + sx : -rx);
+      const T vyn = f == 0 ? -sy : (f == 1 ? ry + sy : -ry);
+      const T inv = rsqrt_fast(mad(vxn, vxn, vyn * vyn));
+      const T nx = vxn * inv, ny = vyn * inv;
+      const T mn = T(-2) * mad(u0[1], nx, u0[2] * ny);
+      un[f][1] = mad(mn, nx, u0[1]);
+      un[f][2] = mad(mn, ny, u0[2]);
     }
-    // neighbour means and dry flags
-    T un[3][4];
-    int dn = 0;
+  }
+  // physical midpoint-minus-centroid vectors from the affine map, up to the Jacobian
+  const T Jd = recip_fast(mad(rx, sy, -(ry * sx)));
+  const T dr[3] = {T(1) / 3, T(1) / 3, T(-2) / 3}, ds[3] = {T(-2) / 3, T(1) / 3, T(1) / 3};
+  const T hb = u0[0] - Bbar;
+  const T cb = sqrt_fast(g * hb), icb = recip_fast(cb), ihb = recip_fast(hb);
+  const T ub = u0[1] * ihb, vb0 = u0[2] * ihb;
+  const T floor = T(1e-6) * mad(sqrt_nn(mad(u0[1], u0[1], u0[2] * u0[2])), icb, hb);
+  const T M = phys_M(p.ph, T(0)), nu = phys_nu(p.ph, T(0));
+  bool changed = false;
+  T dl[3][3];  // limited deltas, [edge][field]
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      const int nb = nbs[f];
-      if (nb >= 0) {
-        dn |= ldm(p.s.dry + nb);
-        load_row_m<T, 4>(p.s.means + 4 * (size_t)nb, un[f]);
-      }
-    }
-    if (de || dn) return;
-    const T rx = gm[0], ry = gm[1], sx = gm[2], sy = gm[3];
-    // a far-field face sees the far-field state over the own mean bed; a wall face
-    // mirrors the normal momentum of the own mean
-    const T Bbar_e = (T)p.s.Bbar[e];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      if (nbs[f] == kFarField) {
-        un[f][0] = (T)p.ph.ff_h + Bbar_e;
-        un[f][1] = (T)p.ph.ff_hu;
-        un[f][2] = (T)p.ph.ff_hv;
-      } else if (nbs[f] < 0) {
-        const T vxn = f == 0 ? -sx : (f == 1 ? rx + sx : -rx);
-        const T vyn = f == 0 ? -sy : (f == 1 ? ry + sy : -ry);
-        const T sn = sqrt(vxn * vxn + vyn * vyn);
-        const T nx = vxn / sn, ny = vyn / sn;
-        const T mn = u0[1] * nx + u0[2] * ny;
-        un[f][0] = u0[0];
-        un[f][1] = u0[1] - T(2) * mn * nx;
-        un[f][2] = u0[2] - T(2) * mn * ny;
-      }
-    }
-    // physical midpoint-minus-centroid vectors from the affine map
-    const T Jd = T(1) / (rx * sy - ry * sx);
-    const T xr = Jd * sy, xs = -Jd * ry, yr = -Jd * sx, ys = Jd * rx;
-    const T dr[3] = {T(1) / 3, T(1) / 3, T(-2) / 3}, ds[3] = {T(-2) / 3, T(1) / 3, T(1) / 3};
-    const T Bbar = Bbar_e;
-    const T hb = u0[0] - Bbar;
-    const T cb = sqrt(g * hb);
-    const T ub = u0[1] / hb, vb0 = u0[2] / hb;
-    const T floor = T(1e-6) * (hb + sqrt(u0[1] * u0[1] + u0[2] * u0[2]) / cb);
-    const T M = (T)p.ph.tvb_M, nu = (T)p.ph.tvb_nu;
-    bool changed = false;
-    T dl[3][3];  // limited deltas, [edge][field]
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const int jj = (cn.w >> (6 + 2 * i)) & 3;
-      const T al = tg[2 * i], be = tg[2 * i + 1];
-      T dt_[3], dn[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        dt_[c] = T(0.5) * (vq[c][i] + vq[c][(i + 1) % 3]) - u0[c];
-        const T uj = jj == 0 ? un[0][c] : (jj == 1 ? un[1][c] : un[2][c]);   // selects, no local array
-        dn[c] = al * (un[i][c] - u0[c]) + be * (uj - u0[c]);
-      }
-      const T mx = xr * dr[i] + xs * ds[i], my = yr * dr[i] + ys * ds[i];
-      const T dist = sqrt(mx * mx + my * my);
-      const T nx = mx / dist, ny = my / dist;
-      // right eigenvectors (columns) and their inverse
-      const T Rm[3][3] = {{T(1), T(0), T(1)},
-                          {ub - cb * nx, -ny, ub + cb * nx},
-                          {vb0 - cb * ny, nx, vb0 + cb * ny}};
-      const T det = Rm[0][0] * (Rm[1][1] * Rm[2][2] - Rm[1][2] * Rm[2][1]) -
-                    Rm[0][1] * (Rm[1][0] * Rm[2][2] - Rm[1][2] * Rm[2][0]) +
-                    Rm[0][2] * (Rm[1][0] * Rm[2][1] - Rm[1][1] * Rm[2][0]);
-      const T id = T(1) / det;
-      T Lm[3][3];
-      Lm[0][0] = (Rm[1][1] * Rm[2][2] - Rm[1][2] * Rm[2][1]) * id;
-      Lm[0][1] = (Rm[0][2] * Rm[2][1] - Rm[0][1] * Rm[2][2]) * id;
-      Lm[0][2] = (Rm[0][1] * Rm[1][2] - Rm[0][2] * Rm[1][1]) * id;
-      Lm[1][0] = (Rm[1][2] * Rm[2][0] - Rm[1][0] * Rm[2][2]) * id;
-      Lm[1][1] = (Rm[0][0] * Rm[2][2] - Rm[0][2] * Rm[2][0]) * id;
-      Lm[1][2] = (Rm[0][2] * Rm[1][0] - Rm[0][0] * Rm[1][2]) * id;
-      Lm[2][0] = (Rm[1][0] * Rm[2][1] - Rm[1][1] * Rm[2][0]) * id;
-      Lm[2][1] = (Rm[0][1] * Rm[2][0] - Rm[0][0] * Rm[2][1]) * id;
-      Lm[2][2] = (Rm[0][0] * Rm[1][1] - Rm[0][1] * Rm[1][0]) * id;
-      const T thr0 = M * dist * dist + floor;
-      T wl[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const T wt = Lm[c][0] * dt_[0] + Lm[c][1] * dt_[1] + Lm[c][2] * dt_[2];
-        const T wn = Lm[c][0] * dn[0] + Lm[c][1] * dn[1] + Lm[c][2] * dn[2];
-        wl[c] = minmod_tvb<T>(wt, nu * wn, c == 1 ? thr0 * cb : thr0, changed);
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) dl[i][c] = Rm[c][0] * wl[0] + Rm[c][1] * wl[1] + Rm[c][2] * wl[2];
-    }
-    if (!changed) return;
-    // redistribution: deltas of each field sum to zero
+  for (int i = 0; i < 3; ++i) {
+    const int jj = (cn.w >> (6 + 2 * i)) & 3;
+    const T al = tg[2 * i], be = tg[2 * i + 1];
+    T dt_[3], dn_[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      T pos = 0, neg = 0;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) { pos += tmax(dl[i][c], T(0)); neg += tmax(-dl[i][c], T(0)); }
-      const T tp = pos > 0 ? tmin(T(1), neg / pos) : T(1);
-      const T tn = neg > 0 ? tmin(T(1), pos / neg) : T(1);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) dl[i][c] = tp * tmax(dl[i][c], T(0)) - tn * tmax(-dl[i][c], T(0));
+      dt_[c] = mad(T(0.5), vq[c][i] + vq[c][(i + 1) % 3], -u0[c]);
+      const T uj = jj == 0 ? un[0][c] : (jj == 1 ? un[1][c] : un[2][c]);   // selects, no local array
+      dn_[c] = mad(al, un[i][c] - u0[c], be * (uj - u0[c]));
     }
-    // depth deltas = eta deltas minus those of Pi1 B; positivity modification (Eq. modified_TVB)
-    T dh[3];
+    const T mx = mad(sy, dr[i], -ry * ds[i]), my = mad(-sx, dr[i], rx * ds[i]);
+    const T m2 = mad(mx, mx, my * my), im = rsqrt_fast(m2);
+    const T nx = mx * im, ny = my * im, dist = Jd * (m2 * im);
+    // characteristic variables: gravity waves (-, +) and shear of the linearised flux
+    // Jacobian in the direction (nx, ny)
+    auto waves = [&](const T (&d)[3], T (&w)[3]) {
+      const T d1 = mad(-ub, d[0], d[1]), d2 = mad(-vb0, d[0], d[2]);
+      const T un_ = mad(d1, nx, d2 * ny) * icb;
+      w[0] = T(0.5) * (d[0] - un_);
+      w[1] = mad(d2, nx, -d1 * ny);
+      w[2] = T(0.5) * (d[0] + un_);
+    };
+    T wt[3], wn[3], wl[3];
+    waves(dt_, wt);
+    waves(dn_, wn);
+    const T thr0 = mad(M * dist, dist, floor);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) dh[i] = dl[i][0] - (T(0.5) * (vb[i] + vb[(i + 1) % 3]) - Bbar);
-    T S[3] = {dh[0] + dh[2] - dh[1], dh[1] + dh[0] - dh[2], dh[2] + dh[1] - dh[0]};
-    const T smin = tmin(S[0], tmin(S[1], S[2]));
-    if (hb + smin < h0) {
-      const T dbar = (dh[0] + dh[1] + dh[2]) / T(3);
-      const T den = dbar - smin;
-      T th = den > 0 ? (hb + dbar - h0) / den : T(1);
-      th = tmin(T(1), tmax(T(0), th));
+    for (int c = 0; c < 3; ++c) wl[c] = minmod_tvb<T>(wt[c], nu * wn[c], c == 1 ? thr0 * cb : thr0, changed);
+    const T sum = wl[0] + wl[2], dif = cb * (wl[2] - wl[0]);
+    dl[i][0] = sum;
+    dl[i][1] = mad(ub, sum, mad(dif, nx, -ny * wl[1]));
+    dl[i][2] = mad(vb0, sum, mad(dif, ny, nx * wl[1]));
+  }
+  if (!changed) return;
+  T vb[3], bb[NP];   // Pi1 B at the vertices, the nodal bed
 #pragma unroll
-      for (int i = 0; i < 3; ++i) dh[i] = dbar + th * (dh[i] - dbar);
-    }
-    // vertex values and the P1 rebuild at the nodes
-    T vh[3], vu[3], vv[3];
-    vh[0] = hb + dh[0] + dh[2] - dh[1]; vh[1] = hb + dh[1] + dh[0] - dh[2]; vh[2] = hb + dh[2] + dh[1] - dh[0];
-    vu[0] = u0[1] + dl[0][1] + dl[2][1] - dl[1][1];
-    vu[1] = u0[1] + dl[1][1] + dl[0][1] - dl[2][1];
-    vu[2] = u0[1] + dl[2][1] + dl[1][1] - dl[0][1];
-    vv[0] = u0[2] + dl[0][2] + dl[2][2] - dl[1][2];
-    vv[1] = u0[2] + dl[1][2] + dl[0][2] - dl[2][2];
-    vv[2] = u0[2] + dl[2][2] + dl[1][2] - dl[0][2];
-    const T* bary = sops + O::BARY;
-    T fld[3][NPP], bb[NPP];
-    load_nodes<T, NP, NPP>(p.s.B + eo, ks, bb);
-    if constexpr (sizeof(T) == 4) {
-      // Single precision: rebuild about the means, eta = eta-bar + sum_v l_v S_v +
-      // (B - B-bar) with S_v the vertex deltas. The stored barycentric weights sum to
-      // one only to rounding (2^-25 at worst), so sum_v l_v (h-bar + S_v) would scale
-      // every rebuilt element's mean by that sum; about the mean the rounding is of
-      // the size of the deltas, not of the depth.
-      const T Sh[3] = {dh[0] + dh[2] - dh[1], dh[1] + dh[0] - dh[2], dh[2] + dh[1] - dh[0]};
-      const T Su[3] = {dl[0][1] + dl[2][1] - dl[1][1], dl[1][1] + dl[0][1] - dl[2][1],
-                       dl[2][1] + dl[1][1] - dl[0][1]};
-      const T Sv[3] = {dl[0][2] + dl[2][2] - dl[1][2], dl[1][2] + dl[0][2] - dl[2][2],
-                       dl[2][2] + dl[1][2] - dl[0][2]};
+  for (int v = 0; v < 3; ++v) vb[v] = __ldg(p.s.vb + v * ks + eo);
 #pragma unroll
-      for (int jn = 0; jn < NP; ++jn) {
-        const T l0 = bary[4 * jn], l1 = bary[4 * jn + 1], l2 = bary[4 * jn + 2];
-        fld[0][jn] = u0[0] + (l0 * Sh[0] + l1 * Sh[1] + l2 * Sh[2]) + (bb[jn] - Bbar);
-        fld[1][jn] = u0[1] + (l0 * Su[0] + l1 * Su[1] + l2 * Su[2]);
-        fld[2][jn] = u0[2] + (l0 * Sv[0] + l1 * Sv[1] + l2 * Sv[2]);
-      }
-    } else {
+  for (int jn = 0; jn < NP; ++jn) bb[jn] = __ldg(p.s.B + eo + jn * ks);
+  // redistribution: deltas of each field sum to zero
 #pragma unroll
-      for (int jn = 0; jn < NP; ++jn) {
-        const T l0 = bary[4 * jn], l1 = bary[4 * jn + 1], l2 = bary[4 * jn + 2];
-        fld[0][jn] = l0 * vh[0] + l1 * vh[1] + l2 * vh[2] + bb[jn];
-        fld[1][jn] = l0 * vu[0] + l1 * vu[1] + l2 * vu[2];
-        fld[2][jn] = l0 * vv[0] + l1 * vv[1] + l2 * vv[2];
-      }
-    }
-    store_nodes<T, NP, NPP>(q + eo, ks, fld[0]);
-    store_nodes<T, NP, NPP>(q + fstride + eo, ks, fld[1]);
-    store_nodes<T, NP, NPP>(q + 2 * fstride + eo, ks, fld[2]);
+  for (int c = 0; c < 3; ++c) {
+    T pos = 0, neg = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) { pos += tmax(dl[i][c], T(0)); neg += tmax(-dl[i][c], T(0)); }
+    const T tp = pos > 0 ? tmin(T(1), neg / pos) : T(1);
+    const T tn = neg > 0 ? tmin(T(1), pos / neg) : T(1);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) dl[i][c] = mad(tp, tmax(dl[i][c], T(0)), -(tn * tmax(-dl[i][c], T(0))));
+  }
+  // depth deltas = eta deltas minus those of Pi1 B; positivity modification (Eq. modified_TVB)
+  T dh[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) dh[i] = dl[i][0] - mad(T(0.5), vb[i] + vb[(i + 1) % 3], -Bbar);
+  // vertex deltas of a field from its midpoint deltas
+  auto vertices = [](const T (&d)[3], T (&S)[3]) {
+    S[0] = d[0] + d[2] - d[1];
+    S[1] = d[1] + d[0] - d[2];
+    S[2] = d[2] + d[1] - d[0];
+  };
+  T S[3];
+  vertices(dh, S);
+  const T smin = tmin(S[0], tmin(S[1], S[2]));
+  if (hb + smin < h0) {
+    const T dbar = (dh[0] + dh[1] + dh[2]) / T(3);
+    const T den = dbar - smin;
+    T th = den > 0 ? (hb + dbar - h0) / den : T(1);
+    th = tmin(T(1), tmax(T(0), th));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) dh[i] = mad(th, dh[i] - dbar, dbar);
+    vertices(dh, S);
+  }
+  const T du[3] = {dl[0][1], dl[1][1], dl[2][1]}, dv[3] = {dl[0][2], dl[1][2], dl[2][2]};
+  T Su[3], Sv[3];
+  vertices(du, Su);
+  vertices(dv, Sv);
+  // the P1 rebuild at the nodes, about the means: eta = eta-bar + sum_v l_v S_v + (B -
+  // B-bar) with S_v the vertex deltas. The stored barycentric weights sum to one only to
+  // rounding, so sum_v l_v (h-bar + S_v) would scale every rebuilt element's mean by that
+  // sum; about the mean the rounding is of the size of the deltas, not of the depth.
+#pragma unroll
+  for (int jn = 0; jn < NP; ++jn) {
+    const T l0 = ops[O::BARY + 4 * jn], l1 = ops[O::BARY + 4 * jn + 1], l2 = ops[O::BARY + 4 * jn + 2];
+    q[jn * ks] = u0[0] + mad(l0, S[0], mad(l1, S[1], l2 * S[2])) + (bb[jn] - Bbar);
+    q[fstride + jn * ks] = u0[1] + mad(l0, Su[0], mad(l1, Su[1], l2 * Su[2]));
+    q[2 * fstride + jn * ks] = u0[2] + mad(l0, Sv[0], mad(l1, Sv[1], l2 * Sv[2]));
   }
 }
 
 // Elements e0, e0 + step, ... below e1 of the TVB limiter (post_stage: 1 limits the
-// just-committed state, 0 the current one). Out of line: the
-// separate launch and the persistent batch kernel then run one compiled copy of its
-// arithmetic (its many short multiply-add chains were rounded differently when it
-// was inlined into the two kernels), at no measured cost.
+// just-committed state, 0 the current one); the separate launch and the persistent batch
+// kernel both inline it.
 template <typename T, int N>
-__device__ __noinline__ void tvb_range(const ScnParams<T>& __restrict__ p, int post_stage,
-                                       const T* __restrict__ sops, int e0, int step, int e1, long long k) {
-  for (int e = e0; e < e1; e += step) tvb_element<T, N>(p, post_stage, sops, e, k);
+__device__ __forceinline__ void tvb_range(const ScnParams<T>& p, int post_stage, const T* ops, int e0, int step, int e1,
+                                          long long k) {
+  for (int e = e0; e < e1; e += step) tvb_element<T, N>(p, post_stage, ops, e, k);
 }
 
 template <typename T, int N>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 3) k_tvb(const __grid_constant__ LimitParams<T> p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sops = reinterpret_cast<T*>(smem_raw);
   if (p.early) dependents_may_launch();
-  stage_ops<T, N, OpLayout<N>::TAIL>(sops, p.s.ops);
   wait_for_previous();
   const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
-  tvb_range<T, N>(p, p.post_stage, sops, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nactive,
+  tvb_range<T, N>(p, p.post_stage, p.s.ops, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, p.nactive,
                   k);
   if (!p.early) dependents_may_launch();
 }

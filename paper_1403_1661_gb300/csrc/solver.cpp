@@ -276,6 +276,9 @@ swe::Phys phys_of(const swe_solver* s, int mask) {
   ph.ff_hv = s->ff[2];
   ph.g_f = (float)ph.g;
   ph.hvel_f = (float)ph.hvel;
+  ph.h0_f = (float)ph.h0;
+  ph.tvb_M_f = (float)ph.tvb_M;
+  ph.tvb_nu_f = (float)ph.tvb_nu;
   ph.ff_h_f = (float)ph.ff_h;
   ph.ff_hu_f = (float)ph.ff_hu;
   ph.ff_hv_f = (float)ph.ff_hv;
