@@ -198,8 +198,14 @@ struct LimitParams : ScnParams<T> {
 
 constexpr int kBatchTile = 128;       // threads per CTA of the SIMT body (four warps, each taking its own
                                       // tickets); the tensor-core body runs the solvers' warps per CTA
-constexpr int kBatchStageTile = 64;   // elements per stage ticket: whole warp-tiles of either body
-constexpr int kBatchTvbTile = 128;    // elements per TVB ticket: four per lane
+// Elements per ticket: one tensor-core tile of the stage phase, one element per lane of
+// the TVB phase. A ticket's elements run one tile after the other on one warp and the next
+// phase waits for the last of them, so the smallest ticket gives the shortest phase: an
+// ensemble of eight scenarios of 5 k to 100 k elements takes 1.34 ms per macro step with
+// tickets of 16, 1.35 with 16 to 64 by phase size, 2.21 with 64.
+constexpr int kBatchStageTile = 16;
+constexpr int kBatchTvbTile = 32;
+constexpr int kBatchCnt = 32;         // ints per scenario in the counter array
 constexpr int kBatchMaxScn = 48;    // scenarios per group launch (kernel-parameter space)
 
 struct alignas(16) BatchSeg {   // one phase of one scenario: tickets [t0, t0 + ntiles)
@@ -212,7 +218,8 @@ struct alignas(16) BatchSeg {   // one phase of one scenario: tickets [t0, t0 + 
   int j;            // substep within the macro step
   int kofs;         // k of this phase minus k at the start of the call
   int first;        // the scenario's first phase in this call: waits for its release
-  int pad[3];
+  int prev;         // tiles of the scenario's phase before this one
+  int pad[2];
 };
 static_assert(sizeof(BatchSeg) == 48, "a segment is three 16-byte words");
 
@@ -234,9 +241,10 @@ struct BatchLaunch {
   const BatchSeg* segs;
   const int* seg_of;  // [tickets] the segment of each ticket
   BatchCtl* ctl;
-  int* done;          // [nscn] tiles completed (run or skipped) per scenario
-  int* ran;           // [nscn] tiles run per scenario
-  int* status;        // [nscn] 0, or SWE_ETIMEOUT when a wait gave up
+  // [nscn] counters, a 128-byte line each (the scenarios' waits poll different lines):
+  // [0] tiles completed (run or skipped), [1] tiles skipped, [2] status: 0, or
+  // SWE_ETIMEOUT when a wait gave up
+  int* cnt;
   const int* release; // [nscn] nonzero: the scenario may start
   int nscn;
   int period[kBatchMaxScn];   // finest substeps per macro step of each scenario

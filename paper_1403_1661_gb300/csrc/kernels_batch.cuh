@@ -1,9 +1,9 @@
 // Persistent batched launch: many scenarios of one (tier, scheme and order) group
 // advanced by one kernel that takes its work from a device ticket queue.
 //
-// A ticket, taken by one warp, is one tile of elements (kBatchStageTile for the stage kernel: R,
-// Adams-Bashforth commit and positivity limiter, Algorithms 1 and 3; kBatchTvbTile
-// for the TVB limiter, Section 5.3) of one phase of one scenario, a phase being one
+// A ticket, taken by one warp, is one tile of elements (kBatchStageTile; the stage kernel: R,
+// Adams-Bashforth commit and positivity limiter, Algorithms 1 and 3;
+// kBatchTvbTile: the TVB limiter, Section 5.3) of one phase of one scenario, a phase being one
 // of those two kernels at one finest substep of the scenario's multirate schedule.
 // Tickets are ordered phase by phase, round-robin over the scenarios (the host builds
 // the segment table), and a ticket runs only after every tile of its scenario's
@@ -41,30 +41,33 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   return v;
 }
 
-// Thread 0 of the CTA: wait until ticket segment S may run. Returns 1 to run the
-// tile, 0 to skip it (its scenario failed, or this wait gave up and failed it).
+// Lane 0 of the warp: wait until ticket segment S may run. Returns 1 to run the tile, 0 to
+// skip it (its scenario failed, or this wait gave up and failed it). A warp may hold a
+// ticket several phases ahead, and a thousand warps polling one counter delay the very
+// updates they wait for: it sleeps 2 us while more than the phase before its own is
+// outstanding, half a microsecond while many tiles of that are, and only then polls fast.
 template <typename T>
 __device__ __forceinline__ int batch_wait(const BatchLaunch<T>& bl, const BatchSeg& S) {
-  const int i = S.scn;
-  if (ld_acquire(bl.status + i) != 0) return 0;
+  int* cnt = bl.cnt + S.scn * kBatchCnt;
+  if (ld_acquire(cnt + 2) != 0) return 0;
   const unsigned long long limit = (unsigned long long)__ldcg(&bl.ctl->wait_ns);
   const unsigned long long t0 = global_ns();
   if (S.first) {
-    while (ld_acquire(bl.release + i) == 0) {
+    while (ld_acquire(bl.release + S.scn) == 0) {
       if (global_ns() - t0 > limit) {
-        atomicCAS(bl.status + i, 0, -5 /* SWE_ETIMEOUT */);
+        atomicCAS(cnt + 2, 0, -5 /* SWE_ETIMEOUT */);
         return 0;
       }
       __nanosleep(256);
     }
   }
-  while (ld_acquire(bl.done + i) < S.need) {
-    if (ld_acquire(bl.status + i) != 0) return 0;
+  for (int rem; (rem = S.need - ld_acquire(cnt)) > 0;) {
+    if (ld_acquire(cnt + 2) != 0) return 0;
     if (global_ns() - t0 > limit) {
-      atomicCAS(bl.status + i, 0, -5 /* SWE_ETIMEOUT */);
+      atomicCAS(cnt + 2, 0, -5 /* SWE_ETIMEOUT */);
       return 0;
     }
-    __nanosleep(64);
+    __nanosleep(rem > S.prev ? 2000 : (rem > 16 ? 500 : 64));
   }
   return 1;
 }
@@ -100,15 +103,15 @@ __device__ __forceinline__ BatchSeg load_seg(const BatchSeg* p) {
 
 // kTC: the tensor-core stage body (FP32 tier); otherwise the SIMT body (T = float
 // or double). Every warp of the CTA takes tickets on its own (no barrier in the
-// loop): a stage ticket is 64 elements (four tensor-core tiles), a TVB ticket 128 elements,
-// four to a lane. Lane 0 holds the warp's next ticket with its segment record,
+// loop). Lane 0 holds the warp's next ticket with its segment record,
 // fetched while the warp works on the current one, and waits only when a ticket
 // opens a segment it has not yet waited for (the tiles a segment needs are the same
 // for all its tickets). The warp prefetches the next stage ticket's node planes to
 // L2, as the separate launch does a tile ahead.
 template <typename T, int N, bool kTC>
 __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k_batch(const __grid_constant__ BatchLaunch<T> bl) {
-  static_assert(kBatchStageTile % 32 == 0 && kBatchTvbTile % 32 == 0, "whole warp-tiles per ticket");
+  static_assert(kBatchStageTile % TcSmem<N>::E == 0 && kBatchStageTile % Team<T, N>::E == 0 && kBatchTvbTile % 32 == 0,
+                "whole warp-tiles per ticket");
   static_assert(sizeof(BatchLaunch<T>) <= 32000, "batch launch parameters exceed the kernel-parameter space");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_k0[kBatchMaxScn];   // finest substep count at the start of the call
@@ -211,8 +214,8 @@ __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k
     __syncwarp();   // the lanes' stores of the tile are issued and ordered before lane 0's
     if (lane == 0) {
       __threadfence();   // ... which a device-scope fence makes visible before the counter moves
-      if (go) atomicAdd(bl.ran + scn, 1);
-      atomicAdd(bl.done + scn, 1);
+      if (!go) atomicAdd(bl.cnt + scn * kBatchCnt + 1, 1);
+      atomicAdd(bl.cnt + scn * kBatchCnt, 1);
     }
   }
 }

@@ -596,7 +596,7 @@ __device__ __forceinline__ double stage_tc_range(const StageParams<float>& __res
   double injected = 0.0;
   int tile = t0;
   do {   // the first pass waits for the operators whether or not the warp has a tile
-    stage_tc_warp<N, kComp>(p, k, nactive, sops, sw, tile, t1, prefetch ? tile + step : -1, first, &injected);
+    stage_tc_warp<N, kComp>(p, k, nactive, sops, sw, tile, t1, prefetch && tile + step < t1 ? tile + step : -1, first, &injected);
     first = false;
     tile += step;
   } while (tile < t1);

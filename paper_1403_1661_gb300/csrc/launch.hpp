@@ -41,8 +41,11 @@ struct Launchers {
   cudaError_t (*split_rhs)(const StageParams<T>&, T* qg, T* rg, const KernelCfg&, cudaStream_t);
   int split_planes;
   // Persistent batch kernel over a group of scenarios of this order (tc: the
-  // tensor-core stage body, FP32 only), grid CTAs.
-  cudaError_t (*batch)(const BatchLaunch<T>& bl, bool tc, int grid, const KernelCfg&, cudaStream_t);
+  // tensor-core stage body, FP32 only), grid CTAs of `warps` warps; beside: sharing the
+  // SMs with other groups' kernels.
+  cudaError_t (*batch)(const BatchLaunch<T>& bl, bool tc, int grid, int warps, bool beside, cudaStream_t);
+  // Registers of one of its warps and shared memory of a CTA of `warps` warps.
+  cudaError_t (*batch_needs)(bool tc, int warps, int* regs_warp, int* smem);
   // Warps per CTA of the tensor-core kernels (FP32 only): sets tc_warps, their
   // shared memory and grids in cfg; cudaErrorInvalidValue when that many warps'
   // tiles do not fit on an SM.
@@ -72,6 +75,25 @@ cudaError_t launch_dependent(void (*kernel)(P...), int blocks, int threads, size
   cudaLaunchAttribute at = {};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Launch a kernel that is to share SMs with others: with the largest shared-memory
+// carve-out, since an SM set up for less does not take a second kernel that needs more
+// until it is empty.
+template <typename... P, typename... A>
+cudaError_t launch_beside(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t st,
+                          const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at.val.sharedMemCarveout = 100;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);

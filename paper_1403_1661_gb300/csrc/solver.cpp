@@ -191,7 +191,8 @@ struct BatchGroup {
   int seg_cap = 0;
   int ticket_cap = 0;
   std::vector<int> seg_of;           // host copy of this call's ticket -> segment table
-  int grid = 0;
+  int grid = 0, warps = 0;           // CTAs of the persistent kernel, warps of each
+  bool beside = false;               // shares the SMs with the other groups' kernels
   cudaStream_t stream = nullptr;     // its branch of the captured graph
   cudaEvent_t join = nullptr;
   std::vector<swe::BatchSeg> segs;   // host copy of this call's ticket segments
@@ -1774,7 +1775,7 @@ int batch_period(const swe_solver* s) { return 1 << (s->L - 1); }
 
 bool batch_tvb(const swe_solver* s) { return (s->prm.limiter_mask & SWE_LIM_TVB) != 0; }
 
-// tickets of one phase: tiles of kBatchStageTile elements (stage) or kBatchTvbTile (TVB)
+// tickets of one phase
 int batch_tiles(int nactive, int kind) {
   const int t = kind == 0 ? swe::kBatchStageTile : swe::kBatchTvbTile;
   return (nactive + t - 1) / t;
@@ -1830,7 +1831,7 @@ size_t batch_layout(std::vector<BatchGroup>& gs, swe_solver* const* solvers, int
     g.off_segs = off;
     off = align256(off + (size_t)cap * sizeof(swe::BatchSeg));
     g.off_cnt = off;
-    off = align256(off + 3 * n * sizeof(int));
+    off = align256(off + swe::kBatchCnt * n * sizeof(int));
     g.off_release = off;
     off = align256(off + n * sizeof(int));
     g.off_nmacro = off;
@@ -1848,7 +1849,7 @@ size_t batch_layout(std::vector<BatchGroup>& gs, swe_solver* const* solvers, int
 void batch_segments(BatchGroup& g, const std::vector<swe_solver*>& solvers, const int32_t* nmacro) {
   g.segs.clear();
   const int n = (int)g.idx.size();
-  std::vector<int> nph(n), need(n, 0);
+  std::vector<int> nph(n), need(n, 0), before(n, 0);   // before: need of the phase before
   int maxp = 0;
   for (int a = 0; a < n; ++a) {
     const swe_solver* s = solvers[g.idx[a]];
@@ -1869,6 +1870,8 @@ void batch_segments(BatchGroup& g, const std::vector<swe_solver*>& solvers, cons
       sg.nactive = s->off[active_levels(s, j)];
       sg.kind = ph % kinds;
       sg.ntiles = batch_tiles(sg.nactive, sg.kind);
+      sg.prev = need[a] - before[a];
+      before[a] = need[a];
       sg.need = need[a];
       sg.scn = a;
       sg.j = j;
@@ -1901,12 +1904,68 @@ swe::BatchLaunch<T> batch_params(const swe_batch* b, const BatchGroup& g) {
   bl.segs = reinterpret_cast<const swe::BatchSeg*>(b->ws + g.off_segs);
   bl.seg_of = reinterpret_cast<const int*>(b->ws + g.off_segof);
   bl.ctl = reinterpret_cast<swe::BatchCtl*>(b->ws + g.off_ctl);
-  bl.done = reinterpret_cast<int*>(b->ws + g.off_cnt);
-  bl.ran = bl.done + n;
-  bl.status = bl.done + 2 * n;
+  bl.cnt = reinterpret_cast<int*>(b->ws + g.off_cnt);
   bl.release = reinterpret_cast<const int*>(b->ws + g.off_release);
   bl.nscn = (int)n;
   return bl;
+}
+
+// Several groups side by side: one CTA of each per SM, its warps in proportion to the
+// group's work as registers and shared memory of an SM allow, so that the groups' chains
+// of dependent phases overlap. (A kernel with a full grid keeps the others off the GPU
+// until it ends.) Groups that do not fit together keep their full grids.
+cudaError_t batch_needs_of(const swe_batch* b, const BatchGroup& g, int warps, int* regs, int* smem) {
+  const swe_solver* s = b->solvers[g.idx[0]];
+  return g.fp64 ? s->ld->batch_needs(g.tc, warps, regs, smem) : s->lf->batch_needs(g.tc, warps, regs, smem);
+}
+
+cudaError_t batch_shares(swe_batch* b, int nsm) {
+  const size_t n = b->groups.size();
+  constexpr int kRegs = 65536, kSmem = 227 * 1024, kReserved = 1024;   // an SM; reserved bytes per CTA
+  std::vector<int> w(n, 1), regs(n);
+  std::vector<double> work(n, 0.0);
+  for (size_t i = 0; i < n; ++i)
+    for (int q : b->groups[i].idx)
+      // the instructions of an element-stage grow like Np times the points per node
+      work[i] += (double)b->dofs[q] * (b->solvers[q]->N + 2) * (b->groups[i].fp64 ? 16 : 1);
+  // Only where phases are short of tickets: with more work than about seven waves of an
+  // all-active phase, full grids (one group after the other) use the GPU better
+  // (per macro step: 28 k elements 0.60 against 0.79 ms, 93 k FP32 0.35 against 0.75, but
+  // 290 k 1.67 against 1.33).
+  int64_t tickets = 0;
+  for (const swe_solver* s : b->solvers) tickets += batch_tiles(s->K, 0);
+  if (tickets > 54 * (int64_t)nsm) return cudaSuccess;
+  auto fits = [&](cudaError_t& err) {
+    int r = 0, m = 0;
+    for (size_t i = 0; i < n; ++i) {
+      int sm = 0;
+      if ((err = batch_needs_of(b, b->groups[i], w[i], &regs[i], &sm))) return false;
+      r += w[i] * regs[i];
+      m += sm + kReserved;
+    }
+    return r <= kRegs && m <= kSmem + kReserved;
+  };
+  cudaError_t err = cudaSuccess;
+  if (!fits(err)) return err;
+  std::vector<char> open(n, 1);
+  for (;;) {   // one more warp to the group with the most work per warp, while it fits
+    int best = -1;
+    for (size_t i = 0; i < n; ++i)
+      if (open[i] && w[i] < b->groups[i].warps && (best < 0 || work[i] / w[i] > work[best] / w[best])) best = (int)i;
+    if (best < 0) break;
+    ++w[best];
+    if (!fits(err)) {
+      if (err) return err;
+      --w[best];
+      open[best] = 0;
+    }
+  }
+  for (size_t i = 0; i < n; ++i) {
+    b->groups[i].warps = w[i];
+    b->groups[i].grid = nsm;
+    b->groups[i].beside = true;
+  }
+  return cudaSuccess;
 }
 
 template <typename T>
@@ -1918,8 +1977,8 @@ cudaError_t batch_enqueue_group(swe_batch* b, const BatchGroup& g) {
   cudaError_t e;
   // a fresh queue: head and the per-scenario counters start at zero
   if ((e = cudaMemsetAsync(b->ws + g.off_ctl, 0, sizeof(int), g.stream))) return e;
-  if ((e = cudaMemsetAsync(b->ws + g.off_cnt, 0, 3 * g.idx.size() * sizeof(int), g.stream))) return e;
-  if ((e = lt->batch(bl, g.tc, g.grid, s0->cfg, g.stream))) return e;
+  if ((e = cudaMemsetAsync(b->ws + g.off_cnt, 0, swe::kBatchCnt * g.idx.size() * sizeof(int), g.stream))) return e;
+  if ((e = lt->batch(bl, g.tc, g.grid, g.warps, g.beside, g.stream))) return e;
   return swe::launch_batch_finish<T>(bl, reinterpret_cast<const int*>(b->ws + g.off_nmacro), g.stream);
 }
 
@@ -1970,10 +2029,8 @@ int swe_batch_create(swe_solver* const* solvers, int32_t n, int32_t max_macro, v
     for (int j = 0; j < batch_period(s); ++j) b->dofs[i] += substep_dofs(s, j);
     b->versions.push_back(s->sched_version);
   }
-  // grids: every group's kernel is given as many CTAs as fit on the GPU; the groups
-  // run side by side and the hardware places their CTAs as room frees up. A CTA takes
-  // tickets only while it is resident, so one that starts late takes fewer, and no
-  // group is held to a share that leaves SMs idle once the others are done.
+  // grids: a single group's kernel is given as many CTAs as fit on the GPU, and so are
+  // several groups whose kernels do not fit on an SM together (batch_shares)
   int dev = 0, nsm = 0;
   SWE_CUDA(cudaGetDevice(&dev));
   SWE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1983,8 +2040,13 @@ int swe_batch_create(swe_solver* const* solvers, int32_t n, int32_t max_macro, v
     const int occ = g.tc ? s0->cfg_max.occ_batch_tc : s0->cfg_max.occ_batch;
     if (occ < 1) return fail(SWE_ECUDA, "the batch kernel does not fit on an SM");
     g.grid = occ * nsm;
+    g.warps = g.tc ? s0->cfg_max.tc_warps : swe::kBatchTile / 32;
     SWE_CUDA(cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking));
     SWE_CUDA(cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming));
+  }
+  if (b->groups.size() > 1) {
+    const cudaError_t se = batch_shares(b.get(), nsm);
+    if (se != cudaSuccess) return fail(SWE_ECUDA, std::string("batch shares: ") + cudaGetErrorString(se));
   }
   SWE_CUDA(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
   SWE_CUDA(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming));
@@ -2083,7 +2145,7 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
   // per scenario: status and tiles run, read back when the step is over
   std::vector<std::vector<int>> host(b->groups.size());
   for (size_t gi = 0; gi < b->groups.size(); ++gi) {
-    host[gi].resize(3 * b->groups[gi].idx.size());
+    host[gi].resize(swe::kBatchCnt * b->groups[gi].idx.size());
     SWE_CUDA(cudaMemcpyAsync(host[gi].data(), b->ws + b->groups[gi].off_cnt, host[gi].size() * sizeof(int),
                              cudaMemcpyDeviceToHost, b->stream));
   }
@@ -2096,7 +2158,8 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
     for (size_t a = 0; a < m; ++a) {
       const int i = g.idx[a];
       swe_solver* s = b->solvers[i];
-      const int st = host[gi][2 * m + a], ran = host[gi][m + a];
+      const int* cnt = &host[gi][swe::kBatchCnt * a];
+      const int st = cnt[2], ran = cnt[0] - cnt[1];
       status_each[i] = st;
       if (st == SWE_OK) {
         s->k += (int64_t)n_macro_each[i] << (s->L - 1);
