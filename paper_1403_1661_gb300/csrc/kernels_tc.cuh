@@ -124,9 +124,9 @@ struct TcSmem {
   // tiles and the fragments fill the shared memory)
   static constexpr int LIMIT = D::N <= 3 ? 12 : (D::N == 4 ? 8 : 7);
   // default warps per CTA (ms per macro step of a 125k-element beach, 45k at N = 5):
-  // N = 2 0.206 (four 0.204, twelve 0.220), N = 3 0.334 (four 0.358, twelve 0.338),
-  // N = 4 0.363 (eight 0.371, two 0.375), N = 5 0.374 (six 0.375, four 0.433)
-  static constexpr int WARPS = D::N <= 3 ? 6 : (D::N == 4 ? 4 : 7);
+  // N = 2 0.180 (six 0.187, eight 0.200), N = 3 0.326 (four 0.357, three 0.364),
+  // N = 4 0.340 (eight 0.350, two 0.352), N = 5 0.355 (six 0.360, four 0.401)
+  static constexpr int WARPS = D::N == 3 ? 6 : (D::N == 5 ? 7 : 4);
 };
 
 // One warp-tile of 16 elements (element e = 16 tile + el). k: the finest substep count;
@@ -143,6 +143,10 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
   using TL = TcLayout<N>;
   using SM = TcSmem<N>;
   constexpr int NP = D::NP, NPP = D::NPP, NFP = D::NFP, KP = C::KP, KSTEP = C::KSTEP, CT = C::CT, NT = C::NT;
+  // Gauss points a lane takes through their chains together (ms per macro step as at
+  // TcSmem::WARPS): one | two at N = 2 0.190 | 0.187 (six warps), N = 3 0.317 | 0.322,
+  // N = 4 0.339 | 0.341, N = 5 0.362 | 0.355
+  constexpr int kPointsAtOnce = D::N == 2 || D::N == 5 ? 2 : 1;
   constexpr bool kBothFaces = D::N == 4;   // registers for both faces' gathers at once
   constexpr int NG = D::NG, KT = C::KT, KF = C::KF, NPT = C::NPT, NB = NPP / 2, BS = SM::BS;
   const uint32_t* sfrag = reinterpret_cast<const uint32_t*>(sops) + SM::FRAG;
@@ -257,29 +261,38 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
         tr[m][3] = add2(make_float2(o[3 * KP * LS], fc.v[3][m]), dup(-Bf));
       }
       const float fr = mad(hu0, vx, hv0 * vy), fu = u0 * fr, fv = v0 * fr;
+      constexpr int G = kPointsAtOnce;   // the last group may repeat the face's last point
 #pragma unroll 1
-      for (int gq = g0; gq < g1; ++gq) {
-        const float* w = sops + OpLayout<N>::I1P + 2 * gq * D::NFPP;
-        float2 te = dup(0.f), tu = te, tv = te, tb = te;
+      for (int gq = g0; gq < g1; gq += G) {
+        float F[G][3];
 #pragma unroll
-        for (int m = 0; m < NFP; m += 2) {
-          float2 wp[2];
-          load4(w + 2 * m, wp);
+        for (int i = 0; i < G; ++i) {
+          const int gi = gq + i < g1 ? gq + i : g1 - 1;
+          const float* w = sops + OpLayout<N>::I1P + 2 * gi * D::NFPP;
+          float2 te = dup(0.f), tu = te, tv = te, tb = te;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            if (m + c >= NFP) continue;
-            te = fma2(wp[c], tr[m + c][0], te);
-            tu = fma2(wp[c], tr[m + c][1], tu);
-            tv = fma2(wp[c], tr[m + c][2], tv);
-            tb = fma2(wp[c], tr[m + c][3], tb);
+          for (int m = 0; m < NFP; m += 2) {
+            float2 wp[2];
+            load4(w + 2 * m, wp);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              if (m + c >= NFP) continue;
+              te = fma2(wp[c], tr[m + c][0], te);
+              tu = fma2(wp[c], tr[m + c][1], tu);
+              tv = fma2(wp[c], tr[m + c][2], tv);
+              tb = fma2(wp[c], tr[m + c][3], tb);
+            }
           }
+          team_flux<float, N>(p.ph, fc.nb, Ef, Bf, E0, B0, nx, ny, hs, vx, vy, te, tu, tv, tb, F[i][0], F[i][1], F[i][2]);
         }
-        float f0, f1, f2;
-        team_flux<float, N>(p.ph, fc.nb, Ef, Bf, E0, B0, nx, ny, hs, vx, vy, te, tu, tv, tb, f0, f1, f2);
-        float* o = sx + (f * NG + gq) * LS + el;
-        o[0] = f0 - fr;
-        o[KF * LS] = f1 - fu;
-        o[2 * KF * LS] = f2 - fv;
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const int gi = gq + i < g1 ? gq + i : g1 - 1;
+          float* o = sx + (f * NG + gi) * LS + el;
+          o[0] = F[i][0] - fr;
+          o[KF * LS] = F[i][1] - fu;
+          o[2 * KF * LS] = F[i][2] - fv;
+        }
       }
     }
   }
