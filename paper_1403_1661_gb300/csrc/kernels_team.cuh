@@ -116,6 +116,10 @@ __device__ __forceinline__ void team_copy(T* dst_, const T* src_) {
   for (int i = threadIdx.x * 16; i < (int)(S * sizeof(T)); i += blockDim.x * 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i), "l"(src + i) : "memory");
 }
+__device__ __forceinline__ void team_copy_ready() {   // the copies of this warp's lanes
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+}
 __device__ __forceinline__ void team_ops_ready() {
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
