@@ -148,7 +148,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-STAGE_KERNEL_SOURCES = ("kernel_types.hpp", "kernels.cuh", "kernels_tc.cuh", "kernels_order.inc")
+STAGE_KERNEL_SOURCES = ("kernel_types.hpp", "kernels.cuh", "kernels_team.cuh", "kernels_tc.cuh", "kernels_order.inc")
 
 
 def kernel_source_hash():
@@ -634,7 +634,7 @@ def run_batched(args, steps=5):
                                   "note": "same solvers and steps, each solver's own captured graph on its own "
                                           "stream, host wall clock"}}
     b.close()
-    # the same batch at the default shape (as many CTAs as fit, four warps per
+    # the same batch at one shape for every order (as many CTAs as fit, four warps per
     # tensor-core CTA): what the tuning buys
     default = {"ctas_per_sm": 0, "tc_warps": 4 if args.precision == "fp32tc" else None}
     for so in solvers:

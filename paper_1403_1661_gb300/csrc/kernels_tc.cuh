@@ -29,13 +29,17 @@
 //
 // What bounds it: latency at two to three warps per scheduler (no pipe is above 25 %,
 // shared memory at half of its wavefronts; more warps cost the registers or the L1 that
-// the gathers need). Per 32 elements at N = 4 it issues 8.5 k warp instructions where
-// the form with 32-element tiles, six interpolated rows, eight projected fluxes and
-// unpacked arithmetic took 11.8 k. Sixteen elements per tile, so that a small active set
-// has twice the tiles and each takes half the time. Measured (GB300), before and after:
-//   one R, 500,000 elements, N = 4                            0.340 -> 0.242 ms
-//   45,149 elements, N = 3, 25 macro steps with transfers      6.39 -> 5.25 ms
-//   2,048 elements, N = 2, 6 macro steps with transfers        0.964 -> 0.788 ms
+// the gathers need: at N = 4 nine warps take 0.42 and ten 0.40 ms per macro step of 125k
+// elements where eight take 0.34). Of a tile's 16 k clocks at N = 4, 2.8 k are the gather,
+// 4.7 k the surface, 4.0 k the volume loop and 1.5 k the commit. Per 32 elements at N = 4
+// it issues 8.5 k warp instructions where the form with 32-element tiles, six interpolated
+// rows, eight projected fluxes and unpacked arithmetic took 11.8 k. Sixteen elements per
+// tile, so that a small active set has twice the tiles and each takes half the time.
+// Measured (GB300, whole calls), before and now, with the overlap of launches and the
+// limiter's shorter form:
+//   one R, 500,000 elements, N = 4                            0.341 -> 0.239 ms
+//   45,149 elements, N = 3, 25 macro steps with transfers      6.42 -> 4.80 ms
+//   2,048 elements, N = 2, 6 macro steps with transfers        0.968 -> 0.608 ms
 #pragma once
 
 #include <cuda_bf16.h>

@@ -38,11 +38,13 @@
 // FP64 instructions, 12.1 k per 32 elements at N = 4 (16.9 k with one thread per element
 // and the six-row form). FP32: the shared-memory pipe (operators arrive at 128 bytes per
 // clock whether they are broadcast or not), then issue slots.
-// Measured (GB300), one thread per element before and this kernel after:
-//   FP64, N = 2, 512 elements, 100 single-rate steps           14.43 -> 2.55 ms
-//   FP64, N = 4, 40,185 elements, 2 macro steps of 4 levels    16.92 -> 9.65 ms
-//   FP32, N = 3, 20,480 elements, 25 limited steps              1.48 -> 1.32 ms
-//   FP32, N = 5, 75,077 elements, one R                        139.7 -> 110.2 us
+// Measured (GB300, whole calls), one thread per element before, and now, with the overlap
+// of launches and the limiter's shorter form, which give the third case half its gain:
+//   FP64, N = 2, 512 elements, 100 single-rate steps           14.45 -> 2.55 ms
+//   FP64, N = 4, 40,185 elements, 2 macro steps of 4 levels    16.95 -> 9.48 ms (93 % of the
+//     FP64 pipe's issue slots in an all-active launch)
+//   FP32, N = 3, 20,480 elements, 25 limited steps              1.47 -> 1.24 ms
+//   FP32, N = 5, 75,077 elements, one R                        140.1 -> 114.6 us
 #pragma once
 
 #include "kernels.cuh"
