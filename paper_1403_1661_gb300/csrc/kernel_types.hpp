@@ -22,6 +22,8 @@ constexpr int kColloc = 16;
 constexpr int kWall = -1;      // reflecting wall
 constexpr int kFarField = -2;  // open: the far-field state of Phys
 constexpr int kReduced = 32;
+// order-code flag of a SIMT stage kernel's variant with sixteen lanes per element
+constexpr int kWide = 64;
 
 template <int NN>
 struct Dims {

@@ -127,16 +127,16 @@ __device__ __forceinline__ void team_ops_ready() {
   __syncthreads();
 }
 
-// Lanes per element and the warp's shared tile. FP64 at N = 2 takes sixteen lanes (its
-// small meshes are bound by the chain of one element: an FP64 instruction holds its
-// warp for 64 cycles), everything else four: NB * L then equals NPP at every order and
-// a quarter-warp's 16-byte reads of eight elements cover all banks (every element
+// Lanes per element and the warp's shared tile. FP64 at N = 2 has a variant with sixteen
+// lanes (kWide; its small meshes are bound by the chain of one element: an FP64
+// instruction holds its warp for 64 cycles; team_wide in kernels_order.inc chooses),
+// everything else takes four: NB * L then equals NPP at every order and a quarter-warp's 16-byte reads of eight elements cover all banks (every element
 // stride is an odd multiple of 16 bytes).
 template <typename T, int N>
 struct Team {
   using D = Dims<N>;
   static constexpr bool FP64 = sizeof(T) == 8;
-  static constexpr int L = FP64 && D::N == 2 ? 16 : 4;
+  static constexpr int L = (N & kWide) ? 16 : 4;
   static constexpr int E = 32 / L;
   static constexpr int NB = D::NPP >= L ? D::NPP / L : 1;   // lanes past NPP have no nodes
   static constexpr int NCH = (D::NCUB + L - 1) / L;   // chunks of L cubature points
@@ -166,8 +166,11 @@ struct Team {
   static constexpr int bytes(int warps) { return (OPS + warps * WARP) * (int)sizeof(T); }
   // warps per CTA when the mesh fills the GPU: eight (two per scheduler), four where
   // their tiles would not fit on an SM (227 KB)
-  static constexpr int MAXW = bytes(8) <= 227 * 1024 ? 8 : 4;
-  // FP32 up to N = 4 runs two CTAs per SM (128 registers), the others one
+  // (FP32 at N = 3 and 4: six, so that two CTAs have 168 registers instead of 128, which
+  // spill: ms per macro step of 125k elements at eight and at six, cubature N = 3 0.357 and
+  // 0.336, N = 4 0.556 and 0.495; one CTA of eight 0.412 and 0.567)
+  static constexpr int MAXW = !FP64 && (D::N == 3 || D::N == 4) ? 6 : (bytes(8) <= 227 * 1024 ? 8 : 4);
+  // FP32 up to N = 4 runs two CTAs per SM, the others one
   static constexpr int MINB = !FP64 && D::N <= 4 ? 2 : 1;
 };
 
@@ -488,6 +491,15 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   using C = Team<T, N>;
   constexpr int NP = D::NP, NPP = D::NPP, NCUB = D::NCUB, E = C::E, NB = C::NB, L = C::L, H = NPP / 2;
   constexpr bool kRegs = sizeof(T) == 4;   // FP32 keeps the interpolated rows in registers
+  // FP32, inexact rules: the reference term -g h0 grad eta is evaluated at the points and
+  // projected with the source (its integrand has degree 2N - 1, which every rule here
+  // integrates exactly), so its derivatives share the rows read for the bed.
+  constexpr bool kFold = kRegs && !D::EXACT;
+  // FP32 collocation: the points are the nodes, so each lane takes its own nodes as its
+  // points. Interpolation and the source's projection are then the identity (nothing to
+  // multiply): with kFold 124 instead of 188 operator reads per lane at N = 4, one R of
+  // 125k elements 0.095 -> 0.078 ms (0.091 with one thread per element).
+  constexpr bool kOwn = kRegs && D::COLLOC;
   const int lane = threadIdx.x & 31, el = lane % E, part = lane / E;
   const int i0 = L * NB == NPP || part < NPP ? part * NB : 0;   // a lane past NPP repeats node 0 (unused)
   const T g = phys_g(p.ph, T(0)), hvel = phys_hvel(p.ph, T(0));
@@ -501,8 +513,10 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
     for (int j = 0; j < NPP; j += 4) {
       Pair<T> ev[2], uv[2], vv[2], bv[2];
       load4(so + j, ev);
-      load4(so + NPP + j, uv);
-      load4(so + 2 * NPP + j, vv);
+      if constexpr (!kOwn) {
+        load4(so + NPP + j, uv);
+        load4(so + 2 * NPP + j, vv);
+      }
       load4(so + 3 * NPP + j, bv);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -512,8 +526,10 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
         if (2 * jj + 1 >= NP) de.y = db.y = T(0);
         s1[jj] = de;
         s0[jj] = D::EXACT ? add2(de, pair(-db.x, -db.y)) : db;
-        s2[jj] = uv[c];
-        s3[jj] = vv[c];
+        if constexpr (!kOwn) {
+          s2[jj] = uv[c];
+          s3[jj] = vv[c];
+        }
       }
     }
   }
@@ -527,27 +543,33 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   for (int f = 0; f < 2; ++f)
 #pragma unroll
     for (int j = 0; j < (kRegs ? H : 1); ++j) M[f][j] = dup(T(0));
+  T own[2][kOwn ? NB : 1];   // collocation: source and reference term of the lane's nodes
+#pragma unroll
+  for (int f = 0; f < 2; ++f)
+#pragma unroll
+    for (int n = 0; n < (kOwn ? NB : 1); ++n) own[f][n] = T(0);
 
 #pragma unroll 1
   for (int ch = 0; ch < C::NCH; ++ch) {
     // interpolation to the lane's point (padding points repeat the last one; FP64 has
     // zero projection weights for them)
-    const int c0 = ch * L + part, c = c0 < NCUB ? c0 : NCUB - 1;
+    const int c0 = kOwn ? i0 + ch : ch * L + part, c = c0 < NCUB ? c0 : NCUB - 1;
     const T* ic = sops + O::IC + c * NPP;
     const T* icr = sops + O::ICR + c * NPP;
     const T* ics = sops + O::ICS + c * NPP;
-    Pair<T> a0 = dup(T(0)), a1 = a0, a2 = a0, a3 = a0, a4 = a0, a5 = a0;
+    Pair<T> a0 = dup(T(0)), a1 = a0, a2 = a0, a3 = a0, a4 = a0, a5 = a0, er = a0, es = a0;
 #pragma unroll
     for (int j = 0; j < NPP; j += 4) {
       Pair<T> w[2], wr[2], ws[2];
-      load4(ic + j, w);
+      if constexpr (!kOwn) load4(ic + j, w);
       load4(icr + j, wr);
       load4(ics + j, ws);
       Pair<T> x0[2], x1[2], x2[2], x3[2];
       if constexpr (kRegs) {
 #pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
-          x0[cc] = s0[j / 2 + cc]; x1[cc] = s1[j / 2 + cc]; x2[cc] = s2[j / 2 + cc]; x3[cc] = s3[j / 2 + cc];
+          x0[cc] = s0[j / 2 + cc]; x1[cc] = s1[j / 2 + cc];
+          if constexpr (!kOwn) { x2[cc] = s2[j / 2 + cc]; x3[cc] = s3[j / 2 + cc]; }
         }
       } else {
         load4(so + 4 * NPP + j, x0);
@@ -558,6 +580,13 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
 #pragma unroll
       for (int cc = 0; cc < 2; ++cc) {
         if (j + 2 * cc >= NP) continue;
+        if constexpr (kOwn) {
+          a4 = fma2(wr[cc], x0[cc], a4);
+          a5 = fma2(ws[cc], x0[cc], a5);
+          er = fma2(wr[cc], x1[cc], er);
+          es = fma2(ws[cc], x1[cc], es);
+          continue;
+        }
         a0 = fma2(w[cc], x0[cc], a0);
         a2 = fma2(w[cc], x2[cc], a2);
         a3 = fma2(w[cc], x3[cc], a3);
@@ -568,10 +597,15 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
           a1 = fma2(w[cc], x1[cc], a1);
           a4 = fma2(wr[cc], x0[cc], a4);
           a5 = fma2(ws[cc], x0[cc], a5);
+          if constexpr (kFold) {
+            er = fma2(wr[cc], x1[cc], er);
+            es = fma2(ws[cc], x1[cc], es);
+          }
         }
       }
     }
-    const T huc = hsum(a2), hvc = hsum(a3), dr = hsum(a4), ds = hsum(a5);
+    const T huc = kOwn ? so[NPP + c] : hsum(a2), hvc = kOwn ? so[2 * NPP + c] : hsum(a3);
+    const T dr = hsum(a4), ds = hsum(a5);
     T hc, F[6];   // rows: Pr (hu, hv), Ps (hu, hv), P (hu, hv)
     const T am = mad(rx, huc, ry * hvc), bm = mad(sx, huc, sy * hvc);
     if constexpr (D::EXACT) {
@@ -582,7 +616,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
       F[4] = gm * mad(rx, dr, sx * ds);
       F[5] = gm * mad(ry, dr, sy * ds);
     } else {
-      const T ec = hsum(a1), bc = hsum(a0);
+      const T ec = kOwn ? so[c] - E0 : hsum(a1), bc = kOwn ? so[3 * NPP + c] - B0 : hsum(a0);
       hc = h0 + (ec - bc);
       const T ih = hc > hvel ? recip_fast(hc) : T(0);
       const T u = huc * ih, v = hvc * ih, gm = -g * ec;
@@ -590,11 +624,16 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
       F[0] = mad(u, am, rx * pr); F[1] = mad(v, am, ry * pr); F[2] = mad(u, bm, sx * pr); F[3] = mad(v, bm, sy * pr);
       F[4] = gm * mad(rx, dr, sx * ds);
       F[5] = gm * mad(ry, dr, sy * ds);
+      if constexpr (kFold) {
+        const T gb = -g * h0, x = hsum(er), y = hsum(es);
+        F[4] = mad(gb, mad(rx, x, sx * y), F[4]);
+        F[5] = mad(gb, mad(ry, x, sy * y), F[5]);
+      }
     }
     if constexpr (kRegs) {   // onto all nodes, padding points excluded
       if (c0 < NCUB) {
 #pragma unroll
-        for (int op = 0; op < 3; ++op) {
+        for (int op = 0; op < (kOwn ? 2 : 3); ++op) {
           const Pair<T> fu = dup(F[2 * op]), fv = dup(F[2 * op + 1]);
           const T* pj = spj + (op * NCUB + c) * NPP;
 #pragma unroll
@@ -607,6 +646,13 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
               M[0][j / 2 + cc] = fma2(w[cc], fu, M[0][j / 2 + cc]);
               M[1][j / 2 + cc] = fma2(w[cc], fv, M[1][j / 2 + cc]);
             }
+          }
+        }
+        if constexpr (kOwn) {
+#pragma unroll
+          for (int n = 0; n < NB; ++n) {
+            own[0][n] = n == ch ? F[4] : own[0][n];
+            own[1][n] = n == ch ? F[5] : own[1][n];
           }
         }
       }
@@ -660,10 +706,21 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   for (int j = 0; j < NPP; j += 4) {
     Pair<T> xa[2], xb[2];
     if constexpr (kRegs) {
+      Pair<T> hu[2], hv[2];
+      if constexpr (kOwn) {
+        load4(so + NPP + j, hu);
+        load4(so + 2 * NPP + j, hv);
+      } else {
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          hu[cc] = s2[j / 2 + cc];
+          hv[cc] = s3[j / 2 + cc];
+        }
+      }
 #pragma unroll
       for (int cc = 0; cc < 2; ++cc) {
-        xa[cc] = fma2(dup(ry), s3[j / 2 + cc], mul2(dup(rx), s2[j / 2 + cc]));
-        xb[cc] = fma2(dup(sy), s3[j / 2 + cc], mul2(dup(sx), s2[j / 2 + cc]));
+        xa[cc] = fma2(dup(ry), hv[cc], mul2(dup(rx), hu[cc]));
+        xb[cc] = fma2(dup(sy), hv[cc], mul2(dup(sx), hu[cc]));
       }
     } else {
       load4(so + 6 * NPP + j, xa);
@@ -703,8 +760,8 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
 #pragma unroll
   for (int f = 0; f < 3; ++f)
 #pragma unroll
-    for (int n = 0; n < NB; ++n) R[f][n] = hsum(A[f][n]);
-  if constexpr (!D::EXACT) {   // strong-form reference pressure (element reference split)
+    for (int n = 0; n < NB; ++n) R[f][n] = f > 0 && kOwn ? hsum(A[f][n]) + own[f > 0 ? f - 1 : 0][kOwn ? n : 0] : hsum(A[f][n]);
+  if constexpr (!D::EXACT && !kFold) {   // strong-form reference pressure (element reference split)
     const T gb = -g * h0;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
@@ -891,37 +948,41 @@ __device__ __forceinline__ void team_commit(const StageParams<T>& p, const T* so
     // element of the warp is wet are the P1 sums taken (FP64 instructions hold a warp
     // for 64 cycles each). Every lane takes part in the sums.
     const double h0 = ph.h0;
-    double hb = 0.0;
+    // The two lane counts of FP64 at N = 2 add up the same tree: P partial sums, a
+    // product each.
+    constexpr int P = sizeof(T) == 8 && D::N == 2 ? 2 : 1;
+    auto total = [](const double (&x)[P]) { return team_sum<L>(P == 2 ? x[0] + x[P - 1] : x[0]); };
+    double hs[P] = {};
 #pragma unroll
     for (int n = 0; n < NB; ++n)
-      if (i0 + n < NP) hb = mad((double)sops[O::MW + ir + n], (double)q[0][n] - (double)q[3][n], hb);
-    hb = team_sum<L>(hb);
+      if (i0 + n < NP)
+        hs[n % P] = mad((double)sops[O::MW + ir + n], (double)q[0][n] - (double)q[3][n], hs[n % P]);
+    const double hb = total(hs);
     const bool isdry = hb < 1.01 * h0;   // the 1% margin keeps a reset element dry under rounding
     if (__any_sync(0xffffffffu, trig && !isdry)) {
-      double ub = 0.0, vb = 0.0;
-      double vh[3] = {0, 0, 0}, vu[3] = {0, 0, 0}, vv[3] = {0, 0, 0};
+      double us[P] = {}, vs[P] = {}, sh[3][P] = {}, su[3][P] = {}, sv[3][P] = {};
 #pragma unroll
       for (int n = 0; n < NB; ++n) {
         if (i0 + n >= NP) continue;
         const double w = (double)sops[O::MW + ir + n];
         const double h = (double)q[0][n] - (double)q[3][n], u = (double)q[1][n], v = (double)q[2][n];
-        ub = mad(w, u, ub);
-        vb = mad(w, v, vb);
+        us[n % P] = mad(w, u, us[n % P]);
+        vs[n % P] = mad(w, v, vs[n % P]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           const double x = (double)sops[O::T1 + k * NPP + ir + n];
-          vh[k] = mad(x, h, vh[k]);
-          vu[k] = mad(x, u, vu[k]);
-          vv[k] = mad(x, v, vv[k]);
+          sh[k][n % P] = mad(x, h, sh[k][n % P]);
+          su[k][n % P] = mad(x, u, su[k][n % P]);
+          sv[k][n % P] = mad(x, v, sv[k][n % P]);
         }
       }
-      ub = team_sum<L>(ub);
-      vb = team_sum<L>(vb);
+      const double ub = total(us), vb = total(vs);
+      double vh[3], vu[3], vv[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        vh[k] = team_sum<L>(vh[k]);
-        vu[k] = team_sum<L>(vu[k]);
-        vv[k] = team_sum<L>(vv[k]);
+        vh[k] = total(sh[k]);
+        vu[k] = total(su[k]);
+        vv[k] = total(sv[k]);
       }
       if (trig && !isdry) {   // theta rescale of the P1 part toward the mean
         const double den = hb - fmin(vh[0], fmin(vh[1], vh[2]));
