@@ -43,7 +43,7 @@
 //   FP64, N = 2, 512 elements, 100 single-rate steps           14.45 -> 2.55 ms
 //   FP64, N = 4, 40,185 elements, 2 macro steps of 4 levels    16.95 -> 9.48 ms (93 % of the
 //     FP64 pipe's issue slots in an all-active launch)
-//   FP32, N = 3, 20,480 elements, 25 limited steps              1.47 -> 1.24 ms
+//   FP32, N = 3, 20,480 elements, 25 limited steps              1.50 -> 1.17 ms
 //   FP32, N = 5, 75,077 elements, one R                        140.1 -> 114.6 us
 #pragma once
 
