@@ -324,10 +324,10 @@ int swe_level_info(const swe_solver* solver, int32_t* L, int32_t* counts, double
  * bit (the same per-element operations; nothing crosses scenarios). */
 typedef struct swe_batch swe_batch;
 
-/* Bytes of caller-owned device workspace (the ticket tables and counters) for a
- * batch of these solvers that advances each by at most max_macro macro steps per
- * swe_batch_step. SWE_EINVAL for NULL arrays, n < 1, max_macro < 1 or a solver
- * without state and levels. */
+/* Bytes of caller-owned device workspace (a 48-byte record per phase, and counters)
+ * for a batch of these solvers that advances each by at most max_macro macro steps
+ * per swe_batch_step. SWE_EINVAL for NULL arrays, n < 1, max_macro < 1, a solver
+ * without state and levels, or a group of more than 2^31 - 1 phases. */
 int swe_batch_workspace_bytes(swe_solver* const* solvers, int32_t n, int32_t max_macro, size_t* bytes);
 
 /* Create a batch of n distinct solvers, each with a valid level-synchronous state

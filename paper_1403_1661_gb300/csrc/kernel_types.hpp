@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <vector_types.h>
 
+#include "batch_tables.hpp"
+
 namespace swe {
 
 constexpr int kMaxLevels = 8;
@@ -200,38 +202,7 @@ struct LimitParams : ScnParams<T> {
 
 constexpr int kBatchTile = 128;       // threads per CTA of the SIMT body (four warps, each taking its own
                                       // tickets); the tensor-core body runs the solvers' warps per CTA
-// Elements per ticket: one tensor-core tile of the stage phase, one element per lane of
-// the TVB phase. A ticket's elements run one tile after the other on one warp and the next
-// phase waits for the last of them, so the smallest ticket gives the shortest phase: an
-// ensemble of eight scenarios of 5 k to 100 k elements takes 1.34 ms per macro step with
-// tickets of 16, 1.35 with 16 to 64 by phase size, 2.21 with 64.
-constexpr int kBatchStageTile = 16;
-constexpr int kBatchTvbTile = 32;
-constexpr int kBatchCnt = 32;         // ints per scenario in the counter array
 constexpr int kBatchMaxScn = 48;    // scenarios per group launch (kernel-parameter space)
-
-struct alignas(16) BatchSeg {   // one phase of one scenario: tickets [t0, t0 + ntiles)
-  int t0;
-  int ntiles;
-  int need;         // tiles of this scenario that must be complete first
-  int scn;          // scenario (index in the group)
-  int nactive;      // active elements
-  int kind;         // 0: stage kernel, 1: TVB limiter
-  int j;            // substep within the macro step
-  int kofs;         // k of this phase minus k at the start of the call
-  int first;        // the scenario's first phase in this call: waits for its release
-  int prev;         // tiles of the scenario's phase before this one
-  int pad[2];
-};
-static_assert(sizeof(BatchSeg) == 48, "a segment is three 16-byte words");
-
-struct BatchCtl {   // per group, in the batch workspace
-  int head;         // next ticket
-  int total;        // tickets of this call
-  int nseg;         // segments of this call
-  int pad;
-  long long wait_ns;  // bound of every wait
-};
 
 template <typename T>
 struct BatchLaunch {
@@ -241,12 +212,8 @@ struct BatchLaunch {
   // read them through the constant cache, which the streaming node data never evicts
   StageParams<T> scn[kBatchMaxScn];
   const BatchSeg* segs;
-  const int* seg_of;  // [tickets] the segment of each ticket
   BatchCtl* ctl;
-  // [nscn] counters, a 128-byte line each (the scenarios' waits poll different lines):
-  // [0] tiles completed (run or skipped), [1] tiles skipped, [2] status: 0, or
-  // SWE_ETIMEOUT when a wait gave up
-  int* cnt;
+  BatchCnt* cnt;      // [nscn]
   const int* release; // [nscn] nonzero: the scenario may start
   int nscn;
   int period[kBatchMaxScn];   // finest substeps per macro step of each scenario

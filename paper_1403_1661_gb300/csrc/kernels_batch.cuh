@@ -40,6 +40,11 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
 
 // Lane 0 of the warp: wait until ticket segment S may run. Returns 1 to run the tile, 0 to
 // skip it (its scenario failed, or this wait gave up and failed it). A warp may hold a
@@ -48,23 +53,23 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 // outstanding, half a microsecond while many tiles of that are, and only then polls fast.
 template <typename T>
 __device__ __forceinline__ int batch_wait(const BatchLaunch<T>& bl, const BatchSeg& S) {
-  int* cnt = bl.cnt + S.scn * kBatchCnt;
-  if (ld_acquire(cnt + 2) != 0) return 0;
+  BatchCnt* cnt = bl.cnt + S.scn;
+  if (ld_acquire(&cnt->status) != 0) return 0;
   const unsigned long long limit = (unsigned long long)__ldcg(&bl.ctl->wait_ns);
   const unsigned long long t0 = global_ns();
   if (S.first) {
     while (ld_acquire(bl.release + S.scn) == 0) {
       if (global_ns() - t0 > limit) {
-        atomicCAS(cnt + 2, 0, -5 /* SWE_ETIMEOUT */);
+        atomicCAS(&cnt->status, 0, -5 /* SWE_ETIMEOUT */);
         return 0;
       }
       __nanosleep(256);
     }
   }
-  for (int rem; (rem = S.need - ld_acquire(cnt)) > 0;) {
-    if (ld_acquire(cnt + 2) != 0) return 0;
+  for (long long rem; (rem = S.need - (long long)ld_acquire(&cnt->done)) > 0;) {
+    if (ld_acquire(&cnt->status) != 0) return 0;
     if (global_ns() - t0 > limit) {
-      atomicCAS(cnt + 2, 0, -5 /* SWE_ETIMEOUT */);
+      atomicCAS(&cnt->status, 0, -5 /* SWE_ETIMEOUT */);
       return 0;
     }
     __nanosleep(rem > S.prev ? 2000 : (rem > 16 ? 500 : 64));
@@ -103,11 +108,11 @@ __device__ __forceinline__ BatchSeg load_seg(const BatchSeg* p) {
 
 // kTC: the tensor-core stage body (FP32 tier); otherwise the SIMT body (T = float
 // or double). Every warp of the CTA takes tickets on its own (no barrier in the
-// loop). Lane 0 holds the warp's next ticket with its segment record,
-// fetched while the warp works on the current one, and waits only when a ticket
-// opens a segment it has not yet waited for (the tiles a segment needs are the same
-// for all its tickets). The warp prefetches the next stage ticket's node planes to
-// L2, as the separate launch does a tile ahead.
+// loop). It holds its next ticket with that ticket's segment record, fetched before the
+// current one runs, and lane 0 waits only when a ticket opens a segment the warp has not
+// yet waited for (the tiles a segment needs are the same for all its tickets). The warp
+// prefetches the next stage ticket's node planes to L2, as the separate launch does a tile
+// ahead.
 template <typename T, int N, bool kTC>
 __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k_batch(const __grid_constant__ BatchLaunch<T> bl) {
   static_assert(kBatchStageTile % TcSmem<N>::E == 0 && kBatchStageTile % Team<T, N>::E == 0 && kBatchTvbTile % 32 == 0,
@@ -130,52 +135,37 @@ __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k
     team_ops_ready();
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int total = __ldcg(&bl.ctl->total);
-  // lane 0: the next ticket and its segment
-  int ticket = 0, nsg = -1, ok_sg = -1;
-  BatchSeg nS;
-  if (lane == 0) {
-    ticket = atomicAdd(&bl.ctl->head, 1);
-    if (ticket < total) {
-      nsg = __ldg(bl.seg_of + ticket);
-      nS = load_seg(bl.segs + nsg);
-    }
-  }
-  for (;;) {
-    // lane 0 takes the held ticket, waits if it opens a segment, and fetches the next
-    int sg = -1, tile = 0, go = 0, scn = 0, kind = 0, nactive = 0, kofs = 0;
-    int pkind = -1, pscn = 0, pe0 = 0, pn = 0, pkofs = 0;   // the next ticket, for the prefetch
-    if (lane == 0 && nsg >= 0) {
-      const BatchSeg S = nS;
-      sg = nsg;
-      tile = ticket - S.t0;
-      scn = S.scn;
-      kind = S.kind;
-      nactive = S.nactive;
-      kofs = S.kofs;
-      go = sg == ok_sg ? 1 : batch_wait(bl, S);
+  const long long total = (long long)__ldcg(&bl.ctl->total);
+  const unsigned nseg = (unsigned)__ldcg(&bl.ctl->nseg);
+  auto take = [&]() {   // the warp's next ticket
+    unsigned long long t = 0;
+    if (lane == 0) t = atomicAdd(&bl.ctl->head, 1ull);
+    return (long long)__shfl_sync(0xffffffffu, t, 0);
+  };
+  // the warp's next ticket and its segment, in every lane
+  long long ticket = take();
+  int sg = 0, ok_sg = -1;
+  BatchSeg S = {};
+  auto find = [&]() {
+    if (ticket < S.t0 + S.ntiles) return;   // still in the segment at hand
+    sg = batch_find((unsigned)sg, nseg, [&](unsigned base, unsigned stride) {
+      const unsigned i = base + lane * stride;
+      return (unsigned)__popc(__ballot_sync(0xffffffffu, i < nseg && __ldg(&bl.segs[i].t0) <= ticket));
+    });
+    S = load_seg(bl.segs + sg);
+  };
+  if (ticket < total) find();
+  while (ticket < total) {
+    // take the held ticket, wait if it opens a segment, and fetch the next
+    const int tile = (int)(ticket - S.t0), scn = S.scn, kind = S.kind, nactive = S.nactive, kofs = S.kofs;
+    int go = 1;
+    if (sg != ok_sg) {
+      if (lane == 0) go = batch_wait(bl, S);
+      go = __shfl_sync(0xffffffffu, go, 0);
       if (go) ok_sg = sg;
-      ticket = atomicAdd(&bl.ctl->head, 1);
-      nsg = -1;
-      if (ticket < total) {
-        nsg = __ldg(bl.seg_of + ticket);
-        nS = load_seg(bl.segs + nsg);
-        pkind = nS.kind;
-        pscn = nS.scn;
-        pe0 = (ticket - nS.t0) * kBatchStageTile;
-        pn = min(kBatchStageTile, nS.nactive - pe0);
-        pkofs = nS.kofs;
-      }
     }
-    sg = __shfl_sync(0xffffffffu, sg, 0);
-    if (sg < 0) break;
-    tile = __shfl_sync(0xffffffffu, tile, 0);
-    go = __shfl_sync(0xffffffffu, go, 0);
-    scn = __shfl_sync(0xffffffffu, scn, 0);
-    kind = __shfl_sync(0xffffffffu, kind, 0);
-    nactive = __shfl_sync(0xffffffffu, nactive, 0);
-    kofs = __shfl_sync(0xffffffffu, kofs, 0);
-    pkind = __shfl_sync(0xffffffffu, pkind, 0);
+    ticket = take();
+    if (ticket < total) find();
     if (go) {
       // the scenario's parameters, in the kernel-parameter space
       const StageParams<T>& wp = bl.scn[scn];
@@ -183,12 +173,9 @@ __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k
       // phase's offset in this call
       const long long k = s_k0[scn] + kofs;
       // the warp's next stage ticket: its planes start moving to L2 now
-      if (pkind == 0) {
-        pscn = __shfl_sync(0xffffffffu, pscn, 0);
-        pe0 = __shfl_sync(0xffffffffu, pe0, 0);
-        pn = __shfl_sync(0xffffffffu, pn, 0);
-        pkofs = __shfl_sync(0xffffffffu, pkofs, 0);
-        batch_prefetch_stage<T, N>(bl.scn[pscn], s_k0[pscn] + pkofs, pe0, pn, lane);
+      if (ticket < total && S.kind == 0) {
+        const int e0 = (int)(ticket - S.t0) * kBatchStageTile;
+        batch_prefetch_stage<T, N>(bl.scn[S.scn], s_k0[S.scn] + S.kofs, e0, min(kBatchStageTile, S.nactive - e0), lane);
       }
       double injected = 0.0;
       if (kind == 0) {
@@ -214,8 +201,8 @@ __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k
     __syncwarp();   // the lanes' stores of the tile are issued and ordered before lane 0's
     if (lane == 0) {
       __threadfence();   // ... which a device-scope fence makes visible before the counter moves
-      if (!go) atomicAdd(bl.cnt + scn * kBatchCnt + 1, 1);
-      atomicAdd(bl.cnt + scn * kBatchCnt, 1);
+      if (!go) atomicAdd(&bl.cnt[scn].skipped, 1ull);
+      atomicAdd(&bl.cnt[scn].done, 1ull);
     }
   }
 }

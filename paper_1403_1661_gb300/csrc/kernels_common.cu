@@ -465,7 +465,7 @@ cudaError_t launch_stats_finalize(const double* partials, int nblocks, double* o
 template <typename T>
 __global__ void k_batch_finish(const __grid_constant__ BatchLaunch<T> bl, const int* n_macro) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < bl.nscn && bl.cnt[i * kBatchCnt + 2] == 0) *bl.scn[i].s.macro += n_macro[i];
+  if (i < bl.nscn && bl.cnt[i].status == 0) *bl.scn[i].s.macro += n_macro[i];
 }
 
 template <typename T>

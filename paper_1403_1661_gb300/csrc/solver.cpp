@@ -187,10 +187,8 @@ struct BatchGroup {
   bool fp64 = false, tc = false;
   int code = 0;
   std::vector<int> idx;              // solvers of the batch in this group
-  size_t off_ctl = 0, off_segs = 0, off_cnt = 0, off_release = 0, off_nmacro = 0, off_segof = 0;
-  int seg_cap = 0;
-  int ticket_cap = 0;
-  std::vector<int> seg_of;           // host copy of this call's ticket -> segment table
+  size_t off_ctl = 0, off_segs = 0, off_cnt = 0, off_release = 0, off_nmacro = 0;
+  int64_t seg_cap = 0;
   int grid = 0, warps = 0;           // CTAs of the persistent kernel, warps of each
   bool beside = false;               // shares the SMs with the other groups' kernels
   cudaStream_t stream = nullptr;     // its branch of the captured graph
@@ -1775,20 +1773,11 @@ int batch_period(const swe_solver* s) { return 1 << (s->L - 1); }
 
 bool batch_tvb(const swe_solver* s) { return (s->prm.limiter_mask & SWE_LIM_TVB) != 0; }
 
-// tickets of one phase
-int batch_tiles(int nactive, int kind) {
-  const int t = kind == 0 ? swe::kBatchStageTile : swe::kBatchTvbTile;
-  return (nactive + t - 1) / t;
-}
-
-// tickets of one macro step of a solver
-int batch_tickets_per_macro(const swe_solver* s) {
-  int n = 0;
-  for (int j = 0; j < batch_period(s); ++j) {
-    const int na = s->off[active_levels(s, j)];
-    n += batch_tiles(na, 0) + (batch_tvb(s) ? batch_tiles(na, 1) : 0);
-  }
-  return n;
+swe::BatchSchedule batch_schedule(const swe_solver* s) {
+  swe::BatchSchedule sc;
+  sc.kinds = batch_tvb(s) ? 2 : 1;
+  for (int j = 0; j < batch_period(s); ++j) sc.nactive.push_back(s->off[active_levels(s, j)]);
+  return sc;
 }
 
 // Group the solvers by precision tier and scheme code, at most kBatchMaxScn per group.
@@ -1813,77 +1802,40 @@ std::vector<BatchGroup> batch_groups(swe_solver* const* solvers, int n) {
 
 // Workspace layout of the batch (each section 256-byte aligned): per group the
 // control block, the ticket segments (capacity for max_macro macro steps of every
-// scenario), the counters done / ran / status (one int each per scenario), the
-// release flags and the macro steps of the call.
-size_t batch_layout(std::vector<BatchGroup>& gs, swe_solver* const* solvers, int max_macro) {
+// scenario), the counters (a BatchCnt per scenario), the release flags and the macro
+// steps of the call. False: more segments than the device indexes.
+bool batch_layout(std::vector<BatchGroup>& gs, swe_solver* const* solvers, int max_macro, size_t* bytes) {
   size_t off = 0;
   for (BatchGroup& g : gs) {
-    int cap = 0, tcap = 0;
-    for (int i : g.idx) {
-      cap += max_macro * batch_period(solvers[i]) * (batch_tvb(solvers[i]) ? 2 : 1);
-      tcap += max_macro * batch_tickets_per_macro(solvers[i]);
-    }
+    int64_t cap = 0;
+    for (int i : g.idx) cap += (int64_t)max_macro * batch_period(solvers[i]) * (batch_tvb(solvers[i]) ? 2 : 1);
+    if (cap > INT32_MAX) return false;
     g.seg_cap = cap;
-    g.ticket_cap = tcap;
     const size_t n = g.idx.size();
     g.off_ctl = off;
     off = align256(off + sizeof(swe::BatchCtl));
     g.off_segs = off;
     off = align256(off + (size_t)cap * sizeof(swe::BatchSeg));
     g.off_cnt = off;
-    off = align256(off + swe::kBatchCnt * n * sizeof(int));
+    off = align256(off + n * sizeof(swe::BatchCnt));
     g.off_release = off;
     off = align256(off + n * sizeof(int));
     g.off_nmacro = off;
     off = align256(off + n * sizeof(int));
-    g.off_segof = off;
-    off = align256(off + (size_t)tcap * sizeof(int));
   }
-  return off;
+  *bytes = off;
+  return true;
 }
 
-// Ticket segments of one call: the phases of every scenario (per macro step and
-// finest substep: the stage kernel, then the TVB limiter), ordered phase by phase,
-// round-robin over the scenarios, each after the tickets of its scenario's earlier
-// phases.
-void batch_segments(BatchGroup& g, const std::vector<swe_solver*>& solvers, const int32_t* nmacro) {
-  g.segs.clear();
-  const int n = (int)g.idx.size();
-  std::vector<int> nph(n), need(n, 0), before(n, 0);   // before: need of the phase before
-  int maxp = 0;
-  for (int a = 0; a < n; ++a) {
-    const swe_solver* s = solvers[g.idx[a]];
-    nph[a] = nmacro[g.idx[a]] * batch_period(s) * (batch_tvb(s) ? 2 : 1);
-    maxp = std::max(maxp, nph[a]);
+// the ticket segments of one call (swe::batch_segments)
+void batch_group_segments(BatchGroup& g, const std::vector<swe_solver*>& solvers, const int32_t* nmacro) {
+  std::vector<swe::BatchSchedule> sc;
+  std::vector<int32_t> nm;
+  for (int i : g.idx) {
+    sc.push_back(batch_schedule(solvers[i]));
+    nm.push_back(nmacro[i]);
   }
-  int t0 = 0;
-  for (int ph = 0; ph < maxp; ++ph)
-    for (int a = 0; a < n; ++a) {
-      if (ph >= nph[a]) continue;
-      const swe_solver* s = solvers[g.idx[a]];
-      const int per = batch_period(s), kinds = batch_tvb(s) ? 2 : 1;
-      const int step = ph / kinds;   // substeps since the start of the call
-      const int j = step % per;
-      swe::BatchSeg sg;
-      std::memset(&sg, 0, sizeof(sg));
-      sg.t0 = t0;
-      sg.nactive = s->off[active_levels(s, j)];
-      sg.kind = ph % kinds;
-      sg.ntiles = batch_tiles(sg.nactive, sg.kind);
-      sg.prev = need[a] - before[a];
-      before[a] = need[a];
-      sg.need = need[a];
-      sg.scn = a;
-      sg.j = j;
-      sg.kofs = step;
-      sg.first = ph == 0 ? 1 : 0;
-      need[a] += sg.ntiles;
-      t0 += sg.ntiles;
-      g.segs.push_back(sg);
-    }
-  g.seg_of.resize(t0);
-  for (size_t q = 0; q < g.segs.size(); ++q)
-    for (int t = 0; t < g.segs[q].ntiles; ++t) g.seg_of[g.segs[q].t0 + t] = (int)q;
+  swe::batch_segments(sc, nm, g.segs);
 }
 
 template <typename T>
@@ -1902,9 +1854,8 @@ swe::BatchLaunch<T> batch_params(const swe_batch* b, const BatchGroup& g) {
   }
   const size_t n = g.idx.size();
   bl.segs = reinterpret_cast<const swe::BatchSeg*>(b->ws + g.off_segs);
-  bl.seg_of = reinterpret_cast<const int*>(b->ws + g.off_segof);
   bl.ctl = reinterpret_cast<swe::BatchCtl*>(b->ws + g.off_ctl);
-  bl.cnt = reinterpret_cast<int*>(b->ws + g.off_cnt);
+  bl.cnt = reinterpret_cast<swe::BatchCnt*>(b->ws + g.off_cnt);
   bl.release = reinterpret_cast<const int*>(b->ws + g.off_release);
   bl.nscn = (int)n;
   return bl;
@@ -1933,7 +1884,7 @@ cudaError_t batch_shares(swe_batch* b, int nsm) {
   // (per macro step: 28 k elements 0.60 against 0.79 ms, 93 k FP32 0.35 against 0.75, but
   // 290 k 1.67 against 1.33).
   int64_t tickets = 0;
-  for (const swe_solver* s : b->solvers) tickets += batch_tiles(s->K, 0);
+  for (const swe_solver* s : b->solvers) tickets += swe::batch_tiles(s->K, 0);
   if (tickets > 54 * (int64_t)nsm) return cudaSuccess;
   auto fits = [&](cudaError_t& err) {
     int r = 0, m = 0;
@@ -1976,8 +1927,8 @@ cudaError_t batch_enqueue_group(swe_batch* b, const BatchGroup& g) {
   const swe::BatchLaunch<T> bl = batch_params<T>(b, g);
   cudaError_t e;
   // a fresh queue: head and the per-scenario counters start at zero
-  if ((e = cudaMemsetAsync(b->ws + g.off_ctl, 0, sizeof(int), g.stream))) return e;
-  if ((e = cudaMemsetAsync(b->ws + g.off_cnt, 0, swe::kBatchCnt * g.idx.size() * sizeof(int), g.stream))) return e;
+  if ((e = cudaMemsetAsync(b->ws + g.off_ctl, 0, sizeof(swe::BatchCtl::head), g.stream))) return e;
+  if ((e = cudaMemsetAsync(b->ws + g.off_cnt, 0, g.idx.size() * sizeof(swe::BatchCnt), g.stream))) return e;
   if ((e = lt->batch(bl, g.tc, g.grid, g.warps, g.beside, g.stream))) return e;
   return swe::launch_batch_finish<T>(bl, reinterpret_cast<const int*>(b->ws + g.off_nmacro), g.stream);
 }
@@ -1991,7 +1942,7 @@ int swe_batch_workspace_bytes(swe_solver* const* solvers, int32_t n, int32_t max
     if (!solvers[i] || !solvers[i]->have_state || !(solvers[i]->dt_min > 0))
       return fail(SWE_EINVAL, "every solver needs state and levels");
   std::vector<BatchGroup> gs = batch_groups(solvers, n);
-  *bytes = batch_layout(gs, solvers, max_macro);
+  if (!batch_layout(gs, solvers, max_macro, bytes)) return fail(SWE_EINVAL, "too many phases in one call: lower max_macro");
   return SWE_OK;
 }
 
@@ -2018,7 +1969,9 @@ int swe_batch_create(swe_solver* const* solvers, int32_t n, int32_t max_macro, v
   b->stream = reinterpret_cast<cudaStream_t>(stream);
   b->max_macro = max_macro;
   b->groups = batch_groups(solvers, n);
-  const size_t need = batch_layout(b->groups, solvers, max_macro);
+  size_t need = 0;
+  if (!batch_layout(b->groups, solvers, max_macro, &need))
+    return fail(SWE_EINVAL, "too many phases in one call: lower max_macro");
   if (bytes < need) return fail(SWE_ENOMEM, "batch workspace smaller than swe_batch_workspace_bytes");
   b->ws = static_cast<char*>(dev_workspace);
   b->ws_bytes = bytes;
@@ -2106,21 +2059,23 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
                        !std::equal(b->last_nmacro.begin(), b->last_nmacro.end(), n_macro_each);
   // this call's tables: ticket segments (when the macro steps changed), the control
   // block, the release flags and the macro steps, uploaded on the batch stream
+  if (rebuild) b->last_nmacro.clear();   // until every group's table is on its way
   for (BatchGroup& g : b->groups) {
     if (rebuild) {
-      batch_segments(g, b->solvers, n_macro_each);
-      if ((int)g.segs.size() > g.seg_cap || (int)g.seg_of.size() > g.ticket_cap)
-        return fail(SWE_EINVAL, "internal: ticket table overflow");
+      try {
+        batch_group_segments(g, b->solvers, n_macro_each);
+      } catch (const std::bad_alloc&) {
+        return fail(SWE_ENOMEM, "host allocation of the ticket segments failed");
+      }
+      if ((int64_t)g.segs.size() > g.seg_cap) return fail(SWE_EINVAL, "internal: segment table overflow");
       if (!g.segs.empty()) {
         SWE_CUDA(cudaMemcpyAsync(b->ws + g.off_segs, g.segs.data(), g.segs.size() * sizeof(swe::BatchSeg),
-                                 cudaMemcpyHostToDevice, b->stream));
-        SWE_CUDA(cudaMemcpyAsync(b->ws + g.off_segof, g.seg_of.data(), g.seg_of.size() * sizeof(int),
                                  cudaMemcpyHostToDevice, b->stream));
       }
     }
     swe::BatchCtl ctl;
     std::memset(&ctl, 0, sizeof(ctl));
-    ctl.total = g.segs.empty() ? 0 : g.segs.back().t0 + g.segs.back().ntiles;
+    ctl.total = g.segs.empty() ? 0 : (unsigned long long)(g.segs.back().t0 + g.segs.back().ntiles);
     ctl.nseg = (int)g.segs.size();
     ctl.wait_ns = (long long)(b->wait_s * 1e9);
     SWE_CUDA(cudaMemcpyAsync(b->ws + g.off_ctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, b->stream));
@@ -2143,10 +2098,10 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
   SWE_CUDA(cudaGraphLaunch(b->graph, b->stream));
   b->launches += 2 * (int64_t)b->groups.size();
   // per scenario: status and tiles run, read back when the step is over
-  std::vector<std::vector<int>> host(b->groups.size());
+  std::vector<std::vector<swe::BatchCnt>> host(b->groups.size());
   for (size_t gi = 0; gi < b->groups.size(); ++gi) {
-    host[gi].resize(swe::kBatchCnt * b->groups[gi].idx.size());
-    SWE_CUDA(cudaMemcpyAsync(host[gi].data(), b->ws + b->groups[gi].off_cnt, host[gi].size() * sizeof(int),
+    host[gi].resize(b->groups[gi].idx.size());
+    SWE_CUDA(cudaMemcpyAsync(host[gi].data(), b->ws + b->groups[gi].off_cnt, host[gi].size() * sizeof(swe::BatchCnt),
                              cudaMemcpyDeviceToHost, b->stream));
   }
   SWE_CUDA(cudaEventRecord(b->done, b->stream));
@@ -2158,8 +2113,8 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
     for (size_t a = 0; a < m; ++a) {
       const int i = g.idx[a];
       swe_solver* s = b->solvers[i];
-      const int* cnt = &host[gi][swe::kBatchCnt * a];
-      const int st = cnt[2], ran = cnt[0] - cnt[1];
+      const swe::BatchCnt& cnt = host[gi][a];
+      const int st = cnt.status;
       status_each[i] = st;
       if (st == SWE_OK) {
         s->k += (int64_t)n_macro_each[i] << (s->L - 1);
@@ -2168,7 +2123,7 @@ int swe_batch_step(swe_batch* b, const int32_t* n_macro_each, int32_t* status_ea
         rc = st;
         // gave up before any of its tiles ran: its state is as before the call;
         // otherwise part of a macro step ran and the state must be set again
-        if (ran > 0) s->have_state = false;
+        if (cnt.done > cnt.skipped) s->have_state = false;
       }
     }
   }
