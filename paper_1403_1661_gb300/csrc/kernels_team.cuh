@@ -25,7 +25,8 @@
 //   pressure and source  the weak pressure p'', its own-side face term, the source
 //             -g eta' grad B' and the strong reference term -g h0 grad eta add up to
 //             the projection of -g h grad eta, which has no cancelling parts at all
-//             (eta = const gives zero). So only h, hu, hv and the two derivatives of
+//             (eta = const gives zero). FP32 projects -g h' grad eta and adds the
+//             reference term as a nodal product (Team::NODAL). So only h, hu, hv and the two derivatives of
 //             eta are interpolated (five rows instead of six), two rows per momentum
 //             carry advection alone and the faces keep only the pressure jump.
 //   mass      hu and hv are polynomials of degree N, so their projection is one
@@ -78,6 +79,14 @@ __device__ __forceinline__ float2 pair(float x, float y) { return make_float2(x,
 __device__ __forceinline__ double2 pair(double x, double y) { return make_double2(x, y); }
 __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
 __device__ __forceinline__ double2 dup(double x) { return make_double2(x, x); }
+// s + a.x b.x + a.y b.y, one after the other. The derivative sums use it: their weights
+// alternate in sign, so the two halves of a packed sum grow large with opposite signs and
+// their difference keeps the rounding of both (R of a bed that varies, FP32 against FP64,
+// rms: 1.1 to 1.75 times that of the plain order, most at N = 5).
+template <typename P, typename T>
+__device__ __forceinline__ T dot2(P a, P b, T s) {
+  return mad(a.y, b.y, mad(a.x, b.x, s));
+}
 template <typename P>
 __device__ __forceinline__ auto hsum(P a) { return a.x + a.y; }
 // four consecutive values (16-byte aligned) as two pairs
@@ -158,8 +167,18 @@ struct Team {
   static constexpr int VF = GEO + (FP64 ? E * GS : 0);
   static constexpr int FX = VF + E * WS;
   static constexpr int WARP = FX + E * XS;            // values per warp
+  // The reference term -g h0 grad eta (h0: the depth at node 0), the leading one at depth: a
+  // nodal product, or evaluated at the points. FP32 keeps it nodal (the points of
+  // collocation are the nodes): through the points it is rounded there and again by the
+  // projection. Rounding of R on a bed that varies, rms over hu and hv against the nodal
+  // form: 1.16 at N = 1, 1.18 at 2, 1.07 at 3, 1.06 at 4, 1.01 at 5; order-2N rules 1.14,
+  // 1.15, 1.12, 1.07 at N = 2 to 5. It costs (ms per macro step of 125k elements, points
+  // and nodal) 0.182 and 0.185, 0.339 and 0.345, 0.497 and 0.514, 0.959 and 0.971 at N = 2
+  // to 5, 0.447 and 0.457 with order-2N rules at N = 4. FP64 with exact rules: no growth
+  // against extended precision, and one product less.
+  static constexpr bool NODAL = FP64 ? !D::EXACT : !D::COLLOC;
   // operators staged per CTA: [0, PRE), then the projection block
-  static constexpr int PRE = D::EXACT ? OpLayout<N>::DR : OpLayout<N>::PRT;
+  static constexpr int PRE = NODAL ? OpLayout<N>::PRT : OpLayout<N>::DR;
   static constexpr int PJ = FP64 ? OpLayout<N>::PROJ4 : OpLayout<N>::PRT;
   static constexpr int NPJ = FP64 ? OpLayout<N>::LGT - OpLayout<N>::PROJ4 : 3 * D::NCUB * D::NPP;
   static constexpr int OPS = PRE + NPJ;
@@ -491,14 +510,12 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   using C = Team<T, N>;
   constexpr int NP = D::NP, NPP = D::NPP, NCUB = D::NCUB, E = C::E, NB = C::NB, L = C::L, H = NPP / 2;
   constexpr bool kRegs = sizeof(T) == 4;   // FP32 keeps the interpolated rows in registers
-  // FP32, inexact rules: the reference term -g h0 grad eta is evaluated at the points and
-  // projected with the source (its integrand has degree 2N - 1, which every rule here
-  // integrates exactly), so its derivatives share the rows read for the bed.
-  constexpr bool kFold = kRegs && !D::EXACT;
+  constexpr bool kNodal = C::NODAL;
   // FP32 collocation: the points are the nodes, so each lane takes its own nodes as its
   // points. Interpolation and the source's projection are then the identity (nothing to
-  // multiply): with kFold 124 instead of 188 operator reads per lane at N = 4, one R of
-  // 125k elements 0.095 -> 0.078 ms (0.091 with one thread per element).
+  // multiply), and the reference term, a nodal product, shares the rows read for the bed:
+  // 124 instead of 188 operator reads per lane at N = 4, one R of 125k elements
+  // 0.095 -> 0.078 ms (0.091 with one thread per element).
   constexpr bool kOwn = kRegs && D::COLLOC;
   const int lane = threadIdx.x & 31, el = lane % E, part = lane / E;
   const int i0 = L * NB == NPP || part < NPP ? part * NB : 0;   // a lane past NPP repeats node 0 (unused)
@@ -557,7 +574,8 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
     const T* ic = sops + O::IC + c * NPP;
     const T* icr = sops + O::ICR + c * NPP;
     const T* ics = sops + O::ICS + c * NPP;
-    Pair<T> a0 = dup(T(0)), a1 = a0, a2 = a0, a3 = a0, a4 = a0, a5 = a0, er = a0, es = a0;
+    Pair<T> a0 = dup(T(0)), a1 = a0, a2 = a0, a3 = a0;
+    T dr = T(0), ds = T(0), er = T(0), es = T(0);
 #pragma unroll
     for (int j = 0; j < NPP; j += 4) {
       Pair<T> w[2], wr[2], ws[2];
@@ -581,38 +599,34 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
       for (int cc = 0; cc < 2; ++cc) {
         if (j + 2 * cc >= NP) continue;
         if constexpr (kOwn) {
-          a4 = fma2(wr[cc], x0[cc], a4);
-          a5 = fma2(ws[cc], x0[cc], a5);
-          er = fma2(wr[cc], x1[cc], er);
-          es = fma2(ws[cc], x1[cc], es);
+          dr = dot2(wr[cc], x0[cc], dr);
+          ds = dot2(ws[cc], x0[cc], ds);
+          er = dot2(wr[cc], x1[cc], er);
+          es = dot2(ws[cc], x1[cc], es);
           continue;
         }
         a0 = fma2(w[cc], x0[cc], a0);
         a2 = fma2(w[cc], x2[cc], a2);
         a3 = fma2(w[cc], x3[cc], a3);
         if constexpr (D::EXACT) {
-          a4 = fma2(wr[cc], x1[cc], a4);
-          a5 = fma2(ws[cc], x1[cc], a5);
+          dr = dot2(wr[cc], x1[cc], dr);
+          ds = dot2(ws[cc], x1[cc], ds);
         } else {
           a1 = fma2(w[cc], x1[cc], a1);
-          a4 = fma2(wr[cc], x0[cc], a4);
-          a5 = fma2(ws[cc], x0[cc], a5);
-          if constexpr (kFold) {
-            er = fma2(wr[cc], x1[cc], er);
-            es = fma2(ws[cc], x1[cc], es);
-          }
+          dr = dot2(wr[cc], x0[cc], dr);
+          ds = dot2(ws[cc], x0[cc], ds);
         }
       }
     }
     const T huc = kOwn ? so[NPP + c] : hsum(a2), hvc = kOwn ? so[2 * NPP + c] : hsum(a3);
-    const T dr = hsum(a4), ds = hsum(a5);
     T hc, F[6];   // rows: Pr (hu, hv), Ps (hu, hv), P (hu, hv)
     const T am = mad(rx, huc, ry * hvc), bm = mad(sx, huc, sy * hvc);
     if constexpr (D::EXACT) {
       hc = h0 + hsum(a0);
       const T ih = hc > hvel ? recip_fast(hc) : T(0);
-      const T u = huc * ih, v = hvc * ih, gm = -g * hc;
+      const T u = huc * ih, v = hvc * ih;
       F[0] = u * am; F[1] = v * am; F[2] = u * bm; F[3] = v * bm;
+      const T gm = -g * (kNodal ? hsum(a0) : hc);   // without or with the reference term
       F[4] = gm * mad(rx, dr, sx * ds);
       F[5] = gm * mad(ry, dr, sy * ds);
     } else {
@@ -624,10 +638,10 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
       F[0] = mad(u, am, rx * pr); F[1] = mad(v, am, ry * pr); F[2] = mad(u, bm, sx * pr); F[3] = mad(v, bm, sy * pr);
       F[4] = gm * mad(rx, dr, sx * ds);
       F[5] = gm * mad(ry, dr, sy * ds);
-      if constexpr (kFold) {
-        const T gb = -g * h0, x = hsum(er), y = hsum(es);
-        F[4] = mad(gb, mad(rx, x, sx * y), F[4]);
-        F[5] = mad(gb, mad(ry, x, sy * y), F[5]);
+      if constexpr (kOwn) {
+        const T gb = -g * h0;
+        F[4] = mad(gb, mad(rx, er, sx * es), F[4]);
+        F[5] = mad(gb, mad(ry, er, sy * es), F[5]);
       }
     }
     if constexpr (kRegs) {   // onto all nodes, padding points excluded
@@ -761,11 +775,11 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   for (int f = 0; f < 3; ++f)
 #pragma unroll
     for (int n = 0; n < NB; ++n) R[f][n] = f > 0 && kOwn ? hsum(A[f][n]) + own[f > 0 ? f - 1 : 0][kOwn ? n : 0] : hsum(A[f][n]);
-  if constexpr (!D::EXACT && !kFold) {   // strong-form reference pressure (element reference split)
+  if constexpr (kNodal) {   // strong-form reference pressure (element reference split)
     const T gb = -g * h0;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
-      Pair<T> er = dup(T(0)), es = er;
+      T er = T(0), es = T(0);
 #pragma unroll
       for (int j = 0; j < NPP; j += 4) {
         Pair<T> wr[2], ws[2], x[2];
@@ -779,12 +793,13 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
         }
 #pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
-          er = fma2(wr[cc], x[cc], er);
-          es = fma2(ws[cc], x[cc], es);
+          if (j + 2 * cc >= NP) continue;
+          er = dot2(wr[cc], x[cc], er);
+          es = dot2(ws[cc], x[cc], es);
         }
       }
-      R[1][n] = mad(gb, mad(rx, hsum(er), sx * hsum(es)), R[1][n]);
-      R[2][n] = mad(gb, mad(ry, hsum(er), sy * hsum(es)), R[2][n]);
+      R[1][n] = mad(gb, mad(rx, er, sx * es), R[1][n]);
+      R[2][n] = mad(gb, mad(ry, er, sy * es), R[2][n]);
     }
   }
 }
