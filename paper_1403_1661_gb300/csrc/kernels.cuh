@@ -142,7 +142,8 @@ __device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
 // Hardware reciprocal and inverse square root without the scaling that the plain calls
 // spend on subnormal arguments (three more instructions each): depths above the dry
-// threshold and squared speeds are normal numbers. FP64: the correctly rounded ones.
+// threshold (Phys::hvel_f is a normal number) and squared speeds are normal numbers. FP64:
+// the correctly rounded ones.
 __device__ __forceinline__ float recip_fast(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -274,7 +275,8 @@ swe::Phys phys_of(const swe_solver* s, int mask) {
   ph.ff_hu = s->ff[1];
   ph.ff_hv = s->ff[2];
   ph.g_f = (float)ph.g;
-  ph.hvel_f = (float)ph.hvel;
+  // the kernels' single-precision reciprocal takes subnormal depths for zero (recip_fast)
+  ph.hvel_f = std::max((float)ph.hvel, std::numeric_limits<float>::min());
   ph.h0_f = (float)ph.h0;
   ph.tvb_M_f = (float)ph.tvb_M;
   ph.tvb_nu_f = (float)ph.tvb_nu;

@@ -30,3 +30,12 @@ def test_fp64_depths_whose_product_underflows(N, scheme):
     a, b = (_rhs("fp64", N, scheme, 0.1 * d, d) / d for d in (1e-100, 1e-170))
     assert np.isfinite(b).all()
     assert np.abs(a - b).max() <= 1e-12 * np.abs(a).max()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32tc"])
+@pytest.mark.parametrize("N,scheme", [(1, "cubature"), (3, "cubature"), (4, "collocation"), (2, "cubature_2n")])
+def test_fp32_subnormal_depths(precision, N, scheme):
+    # a film of subnormal depth over a subnormal threshold: no velocity, and no infinity from
+    # a reciprocal that takes such a depth for zero
+    R = _rhs(precision, N, scheme, 2e-39, 5e-39)
+    assert np.isfinite(R).all()
