@@ -511,6 +511,12 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   // 124 instead of 188 operator reads per lane at N = 4, one R of 125k elements
   // 0.095 -> 0.078 ms (0.091 with one thread per element).
   constexpr bool kOwn = kRegs && D::COLLOC;
+  // FP64 collocation uses the same identities on the team's common points: a lane's point is
+  // read from the tile, and the source comes back to the lane of its node. ms per macro step
+  // with the points interpolated and projected as of the other schemes, and so: N = 2, 80k
+  // elements 2.66 and 2.46 (2.47 with one thread per element), 20k elements N = 2 0.91 and
+  // 0.85, N = 4 1.76 and 1.49, N = 5 3.02 and 2.43.
+  constexpr bool kIdent = D::COLLOC;
   const int lane = threadIdx.x & 31, el = lane % E, part = lane / E;
   const int i0 = L * NB == NPP || part < NPP ? part * NB : 0;   // a lane past NPP repeats node 0 (unused)
   const T g = phys_g(p.ph, T(0)), hvel = phys_hvel(p.ph, T(0));
@@ -554,11 +560,11 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
   for (int f = 0; f < 2; ++f)
 #pragma unroll
     for (int j = 0; j < (kRegs ? H : 1); ++j) M[f][j] = dup(T(0));
-  T own[2][kOwn ? NB : 1];   // collocation: source and reference term of the lane's nodes
+  T own[2][kIdent ? NB : 1];   // collocation: source (FP32: and reference term) of the lane's nodes
 #pragma unroll
   for (int f = 0; f < 2; ++f)
 #pragma unroll
-    for (int n = 0; n < (kOwn ? NB : 1); ++n) own[f][n] = T(0);
+    for (int n = 0; n < (kIdent ? NB : 1); ++n) own[f][n] = T(0);
 
 #pragma unroll 1
   for (int ch = 0; ch < C::NCH; ++ch) {
@@ -573,7 +579,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
 #pragma unroll
     for (int j = 0; j < NPP; j += 4) {
       Pair<T> w[2], wr[2], ws[2];
-      if constexpr (!kOwn) load4(ic + j, w);
+      if constexpr (!kIdent) load4(ic + j, w);
       load4(icr + j, wr);
       load4(ics + j, ws);
       Pair<T> x0[2], x1[2], x2[2], x3[2];
@@ -585,18 +591,22 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
         }
       } else {
         load4(so + 4 * NPP + j, x0);
-        load4(so + 5 * NPP + j, x1);
-        load4(so + NPP + j, x2);
-        load4(so + 2 * NPP + j, x3);
+        if constexpr (!kIdent) {
+          load4(so + 5 * NPP + j, x1);
+          load4(so + NPP + j, x2);
+          load4(so + 2 * NPP + j, x3);
+        }
       }
 #pragma unroll
       for (int cc = 0; cc < 2; ++cc) {
         if (j + 2 * cc >= NP) continue;
-        if constexpr (kOwn) {
+        if constexpr (kIdent) {
           dr = dot2(wr[cc], x0[cc], dr);
           ds = dot2(ws[cc], x0[cc], ds);
-          er = dot2(wr[cc], x1[cc], er);
-          es = dot2(ws[cc], x1[cc], es);
+          if constexpr (kOwn) {
+            er = dot2(wr[cc], x1[cc], er);
+            es = dot2(ws[cc], x1[cc], es);
+          }
           continue;
         }
         a0 = fma2(w[cc], x0[cc], a0);
@@ -612,7 +622,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
         }
       }
     }
-    const T huc = kOwn ? so[NPP + c] : hsum(a2), hvc = kOwn ? so[2 * NPP + c] : hsum(a3);
+    const T huc = kIdent ? so[NPP + c] : hsum(a2), hvc = kIdent ? so[2 * NPP + c] : hsum(a3);
     T hc, F[6];   // rows: Pr (hu, hv), Ps (hu, hv), P (hu, hv)
     const T am = mad(rx, huc, ry * hvc), bm = mad(sx, huc, sy * hvc);
     if constexpr (D::EXACT) {
@@ -624,7 +634,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
       F[4] = gm * mad(rx, dr, sx * ds);
       F[5] = gm * mad(ry, dr, sy * ds);
     } else {
-      const T ec = kOwn ? so[c] - E0 : hsum(a1), bc = kOwn ? so[3 * NPP + c] - B0 : hsum(a0);
+      const T ec = kIdent ? so[c] - E0 : hsum(a1), bc = kIdent ? so[3 * NPP + c] - B0 : hsum(a0);
       hc = h0 + (ec - bc);
       const T ih = hc > hvel ? recip_fast(hc) : T(0);
       const T u = huc * ih, v = hvc * ih, gm = -g * ec;
@@ -679,7 +689,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
 #pragma unroll
         for (int n = 0; n < NB; ++n)
 #pragma unroll
-          for (int op = 0; op < 3; ++op) {
+          for (int op = 0; op < (kIdent ? 2 : 3); ++op) {
             Pair<T> w[2];
             load4(pj + (op * NPP + n) * 4, w);
 #pragma unroll
@@ -687,6 +697,14 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
               A[1][n] = fma2(w[cc], x[2 * op][cc], A[1][n]);
               A[2][n] = fma2(w[cc], x[2 * op + 1][cc], A[2][n]);
             }
+          }
+      }
+      if constexpr (kIdent) {   // the source at the lane's nodes among these points
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+          if (i0 + n < NP && (i0 + n) / L == ch) {
+            own[0][n] = vf[4 * L + (i0 + n) % L];
+            own[1][n] = vf[5 * L + (i0 + n) % L];
           }
       }
       __syncwarp();
@@ -768,7 +786,7 @@ __device__ __forceinline__ void team_rhs(const StageParams<T>& p, const T* sops,
 #pragma unroll
   for (int f = 0; f < 3; ++f)
 #pragma unroll
-    for (int n = 0; n < NB; ++n) R[f][n] = f > 0 && kOwn ? hsum(A[f][n]) + own[f > 0 ? f - 1 : 0][kOwn ? n : 0] : hsum(A[f][n]);
+    for (int n = 0; n < NB; ++n) R[f][n] = f > 0 && kIdent ? hsum(A[f][n]) + own[f > 0 ? f - 1 : 0][kIdent ? n : 0] : hsum(A[f][n]);
   if constexpr (kNodal) {   // strong-form reference pressure (element reference split)
     const T gb = -g * h0;
 #pragma unroll
