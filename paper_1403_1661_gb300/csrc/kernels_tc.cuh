@@ -213,7 +213,7 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
 #pragma unroll
       for (int pl = 0; pl < 3 * NP; pl += 32)
         if (pl + lane < 3 * NP) {
-          const unsigned o = (unsigned)(pl + lane) * (unsigned)sc.KS;
+          const size_t o = (size_t)(pl + lane) * sc.KS;   // 3 NP planes: past 2^32 words on the largest meshes
           prefetch_l2(ra + o);
           prefetch_l2(rb + o);
           if constexpr (kComp) prefetch_l2(p.s.comp + e0 + o);
@@ -226,8 +226,8 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
       const float* bn = p.s.B + e0;
 #pragma unroll
       for (int pl = 0; pl < 3 * NP; pl += 32)
-        if (pl + lane < 3 * NP) prefetch_l2(qn + (unsigned)(pl + lane) * (unsigned)sc.KS);
-      if (lane < NP) prefetch_l2(bn + (unsigned)lane * (unsigned)sc.KS);
+        if (pl + lane < 3 * NP) prefetch_l2(qn + (size_t)(pl + lane) * sc.KS);
+      if (lane < NP) prefetch_l2(bn + (size_t)lane * sc.KS);
     }
     if (first) team_ops_ready();
     if (tile >= ntiles) return;
