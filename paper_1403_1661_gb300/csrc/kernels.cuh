@@ -244,8 +244,8 @@ __host__ __device__ constexpr int face_node(int N, int f, int m) {
 __device__ __forceinline__ int face_node_rt(int N, int f, int m) { return face_node(N, f, m); }
 
 // Stage the first S entries of the operator block into shared memory (all threads
-// of the CTA): the whole block for the SIMT stage kernel, the per-element
-// operators [0, TAIL) for the limiter kernels.
+// of the CTA): the whole block for the kernel-split ablation, the per-element
+// operators [0, TAIL) for the positivity kernel and the ablation's traces.
 template <typename T, int N, int S = OpLayout<N>::SIZE>
 __device__ __forceinline__ void stage_ops(T* sops, const T* __restrict__ gops) {
   using V = Vec16<T>;

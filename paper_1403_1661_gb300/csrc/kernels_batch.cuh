@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kTC ? 32 * TcSmem<N>::LIMIT : kBatchTile, 1) k
           float* sw = sops + SM::CTA + warp * SM::WARP;
           const int t0 = tile * (kBatchStageTile / SM::E);
           const int t1 = min(t0 + kBatchStageTile / SM::E, (nactive + SM::E - 1) / SM::E);
-          injected = stage_tc_range<N>(wp, k, nactive, sops, sw, t0, 1, t1, true, false);
+          injected = stage_tc_range<N>(wp, k, nactive, sops, sw, t0, 1, t1, false);
         } else {
           using C = Team<T, N>;
           T* sw = sops + C::OPS + warp * C::WARP;

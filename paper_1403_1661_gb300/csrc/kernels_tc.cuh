@@ -27,7 +27,7 @@
 // The operators' fragments are staged once per CTA in shared memory; results do not
 // depend on the number of warps per CTA.
 //
-// What bounds it: latency at two to three warps per scheduler (no pipe is above 25 %,
+// What bounds it: latency at two to three warps per scheduler (no pipe is above 27 %,
 // shared memory at half of its wavefronts; more warps cost the registers or the L1 that
 // the gathers need: at N = 4 nine warps take 0.42 and ten 0.40 ms per macro step of 125k
 // elements where eight take 0.34). Of a tile's 16 k clocks at N = 4, 2.8 k are the gather,
@@ -124,9 +124,9 @@ struct TcSmem {
   static constexpr int CTA = OPS + TcLayout<N>::SIZE;     // floats per CTA before the warps' tiles
   // dynamic shared memory of a CTA of `warps` warps
   static constexpr int bytes(int warps) { return (CTA + warps * WARP) * 4; }
-  // warps per SM the registers are budgeted for, as many as a CTA may have: twelve up to
-  // N = 3 (168 registers), eight at N = 4 (255; twelve spill), seven at N = 5 (their
-  // tiles and the fragments fill the shared memory)
+  // warps per SM the registers are budgeted for: twelve up to N = 3 (168 registers), eight
+  // at N = 4 (255; twelve spill), seven at N = 5 (their tiles and the fragments fill the
+  // shared memory). A CTA has at most eight (swe_set_tc_warps)
   static constexpr int LIMIT = D::N <= 3 ? 12 : (D::N == 4 ? 8 : 7);
   // default warps per CTA (ms per macro step of a 125k-element beach, 45k at N = 5):
   // N = 2 0.180 (six 0.187, eight 0.200), N = 3 0.326 (four 0.357, three 0.364),
@@ -153,7 +153,10 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
   // TcSmem::WARPS): one | two at N = 2 0.190 | 0.187 (six warps), N = 3 0.317 | 0.322,
   // N = 4 0.339 | 0.341, N = 5 0.362 | 0.355
   constexpr int kPointsAtOnce = D::N == 2 || D::N == 5 ? 2 : 1;
-  constexpr bool kBothFaces = D::N == 4;   // registers for both faces' gathers at once
+  // both faces' gathers at once, or the second after the first face's fluxes (ms per macro
+  // step of a 125k-element beach, 45k at N = 5): N = 3 0.384 and 0.358, N = 4 0.363 and 0.376,
+  // N = 5 0.427 (spills) and 0.374
+  constexpr bool kBothFaces = D::N == 4;
   constexpr int NG = D::NG, KT = C::KT, KF = C::KF, NPT = C::NPT, NB = NPP / 2, BS = SM::BS;
   const uint32_t* sfrag = reinterpret_cast<const uint32_t*>(sops) + SM::FRAG;
   const int lane = threadIdx.x & 31;
@@ -619,20 +622,20 @@ __device__ __forceinline__ void stage_tc_init(float* sw) {
   __syncwarp();
 }
 
-// Warp-tiles t0, t0 + step, ... below t1 (each warp calls it for its own tiles; with
-// prefetch the planes of the warp's next tile are prefetched to L2); returns the mass
-// the positivity limiter's dry resets injected. The separate launch and the persistent
+// Warp-tiles t0, t0 + step, ... below t1 (each warp calls it for its own tiles; the planes
+// of its next tile are prefetched to L2); returns the mass the positivity limiter's dry
+// resets injected. The separate launch and the persistent
 // batch kernel both inline it (out of line the body ran 1.5 times slower: its parameters
 // become memory loads).
 template <int N, bool kComp = false>
 __device__ __forceinline__ double stage_tc_range(const StageParams<float>& __restrict__ p, long long k,
                                               int nactive, const float* __restrict__ sops, float* sw, int t0,
-                                              int step, int t1, bool prefetch, bool first) {
+                                              int step, int t1, bool first) {
   double injected = 0.0;
   int tile = t0;
   bool have = false;
   do {   // the first pass waits for the operators whether or not the warp has a tile
-    const bool next = prefetch && tile + step < t1;
+    const bool next = tile + step < t1;
     stage_tc_warp<N, kComp>(p, k, nactive, sops, sw, tile, t1, next ? tile + step : -1, first, have, &injected);
     first = false;
     have = next;
@@ -650,7 +653,7 @@ __device__ __forceinline__ void tc_ops_begin(float* smem, const float* ops, cons
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// CTA: blockDim.x / 32 warps (1 to MAXW), each with its own shared tiles after the CTA's
+// CTA: blockDim.x / 32 warps (1 to 8, swe_set_tc_warps), each with its own shared tiles after the CTA's
 // operators. kComp: compensated state update (p.s.comp).
 template <int N, bool kComp = false>
 __global__ void __launch_bounds__(32 * TcSmem<N>::LIMIT, 1) k_stage_tc(const __grid_constant__ StageParams<float> p) {
@@ -666,7 +669,7 @@ __global__ void __launch_bounds__(32 * TcSmem<N>::LIMIT, 1) k_stage_tc(const __g
   const long long k = (*p.s.macro) * (1LL << (p.sc.L - 1)) + p.j;
   const int ntiles = (p.nactive + SM::E - 1) / SM::E;
   const double injected =
-      stage_tc_range<N, kComp>(p, k, p.nactive, sops, sw, blockIdx.x * nw + warp, gridDim.x * nw, ntiles, true, true);
+      stage_tc_range<N, kComp>(p, k, p.nactive, sops, sw, blockIdx.x * nw + warp, gridDim.x * nw, ntiles, true);
   if (!p.early) dependents_may_launch();
   if (injected != 0.0) atomicAdd(p.s.acc, injected);
 }

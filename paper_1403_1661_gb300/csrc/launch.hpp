@@ -16,12 +16,12 @@ struct KernelCfg {
   int smem_bytes = 0;      // the whole operator block (kernel-split ablation)
   int smem_lim = 0;        // the per-element operators (limiter kernels)
   int grid_stage = 0, grid_pos = 0, grid_tvb = 0, grid_stats = 0;
-  int smem_tc = 0, grid_tc = 0;   // tensor-core stage kernel (FP32 only)
+  int grid_tc = 0;                // tensor-core stage kernel (FP32 only)
   int tc_warps = 4;               // warps per CTA of the tensor-core stage and batch kernels
   int grid_stage_g = 0;           // stage kernel with the operators in global memory
   int grid_split_t = 0, grid_split_v = 0, grid_split_s = 0;   // kernel-split ablation
-  int smem_batch = 0, occ_batch = 0;         // persistent batch kernel, SIMT body
-  int smem_batch_tc = 0, occ_batch_tc = 0;   // persistent batch kernel, tensor-core body (FP32)
+  int occ_batch = 0;              // persistent batch kernel, SIMT body
+  int occ_batch_tc = 0;           // persistent batch kernel, tensor-core body (FP32)
 };
 
 template <typename T>
