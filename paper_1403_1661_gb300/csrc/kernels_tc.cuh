@@ -206,7 +206,10 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
       }
     }
     // this tile's older R slots and the next tile's planes start moving now (hints; the
-    // first element's level stands for the tile)
+    // first element's level stands for the tile). 64-bit offsets: the planes of three fields
+    // pass 2^32 words above 97 million elements at N = 4 (one wide product per lane; a wide
+    // product per plane took 0.6 % of R at N = 4 and 1.5 % of a macro step at N = 5)
+    const size_t lane_ks = (size_t)(unsigned)lane * (unsigned)sc.KS;
     if (p.mode == 0 && tile < ntiles) {
       const int e0 = tile * 16;
       const long long a0 = __shfl_sync(0xffffffffu, a, 0);
@@ -216,7 +219,7 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
 #pragma unroll
       for (int pl = 0; pl < 3 * NP; pl += 32)
         if (pl + lane < 3 * NP) {
-          const size_t o = (size_t)(pl + lane) * sc.KS;   // 3 NP planes: past 2^32 words on the largest meshes
+          const size_t o = lane_ks + (size_t)pl * sc.KS;
           prefetch_l2(ra + o);
           prefetch_l2(rb + o);
           if constexpr (kComp) prefetch_l2(p.s.comp + e0 + o);
@@ -229,8 +232,8 @@ __device__ __forceinline__ void stage_tc_warp(const StageParams<float>& p, long 
       const float* bn = p.s.B + e0;
 #pragma unroll
       for (int pl = 0; pl < 3 * NP; pl += 32)
-        if (pl + lane < 3 * NP) prefetch_l2(qn + (size_t)(pl + lane) * sc.KS);
-      if (lane < NP) prefetch_l2(bn + (size_t)lane * sc.KS);
+        if (pl + lane < 3 * NP) prefetch_l2(qn + (size_t)pl * sc.KS + lane_ks);
+      if (lane < NP) prefetch_l2(bn + lane_ks);
     }
     if (first) team_ops_ready();
     if (tile >= ntiles) return;
