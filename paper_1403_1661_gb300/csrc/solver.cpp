@@ -17,6 +17,7 @@
 #include "launch.hpp"
 #include "mesh.hpp"
 #include "refelem.hpp"
+#include "split_bf16.hpp"
 
 struct swe_mesh {
   swe::Mesh m;
@@ -298,18 +299,6 @@ std::vector<T> to_t(const std::vector<double>& v) {
   return o;
 }
 
-// bf16 round-to-nearest-even of a float (host), and its value
-uint16_t bf16_bits(float f) {
-  uint32_t u;
-  std::memcpy(&u, &f, 4);
-  return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
-}
-float bf16_value(uint16_t b) {
-  uint32_t u = (uint32_t)b << 16;
-  float f;
-  std::memcpy(&f, &u, 4);
-  return f;
-}
 // hi/lo TF32 split of an operator entry: hi rounded to 10 mantissa bits (to
 // nearest, ties away), lo = the single-precision remainder (the tensor core reads
 // its top 10 mantissa bits)
@@ -323,13 +312,6 @@ void tf32_split(double v, uint32_t& hi, uint32_t& lo) {
   const float l = vf - h;
   hi = u;
   std::memcpy(&lo, &l, 4);
-}
-
-// hi/lo bf16 split of a single-precision operator entry
-void bf16_split(double v, uint16_t& hi, uint16_t& lo) {
-  const float vf = (float)v;
-  hi = bf16_bits(vf);
-  lo = bf16_bits(vf - bf16_value(hi));
 }
 
 // Pack the FP64 reference operators into the kernels' operator block (OpLayout)
@@ -400,6 +382,31 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
   put_rows(O::PST, e.Ps, nc, np, true);
   put_rows(O::PT, e.P, nc, np, true);
 
+  // The mass operator as the tensor cores hold it, rounded for fields that are linear and,
+  // with a tenth of the weight, quadratic in an element (relative to node 0, as the kernel
+  // takes them). Error of hu and hv after 8 macro steps of a beach of 20,000 elements against
+  // 64 bits, with low parts to nearest and so, in parts of that of products at the points (the
+  // form before there was a nodal mass operator): N = 3 0.91, 1.14 and 0.81, 0.88; N = 4 0.97,
+  // 0.75 and 0.93, 0.73; N = 5 0.86, 1.06 and 0.82, 0.81; order-2N rules N = 3 1.18, 1.35 and
+  // 0.73, 0.70, N = 4 1.10, 1.18 and 0.99, 1.13 (1.04 with TF32 products, 2^-21, for 4 to 12 %
+  // of a macro step: what is left there is not this operator's).
+  // Collocation keeps the nearest values: its Pr, Ps are this operator too.
+  std::vector<double> mass[2];
+  {
+    std::vector<std::vector<double>> modes(5);
+    for (int j = 0; j < np; ++j) {
+      const double x = e.r[j] - e.r[0], y = e.s[j] - e.s[0];
+      const double f[5] = {x, y, 0.1 * x * x, 0.1 * x * y, 0.1 * y * y};
+      for (int q = 0; q < 5; ++q) modes[q].push_back(f[q]);
+    }
+    for (int op = 0; op < 2; ++op)
+      for (int i = 0; i < np; ++i) {
+        const double* w = &o[(op == 0 ? O::WR : O::WS) + (size_t)i * npp];
+        const std::vector<double> r = D::COLLOC ? std::vector<double>(w, w + np) : swe::smooth_row(w, np, modes);
+        mass[op].insert(mass[op].end(), r.begin(), r.end());
+      }
+  }
+
   // tensor-core fragments (mma.sync m16n8k16 / m16n8k8 bf16 B operands): lane (g, t)
   // holds column n = g, rows k = 2t, 2t+1 (and 2t+8, 2t+9)
   tc.assign(TL::SIZE, 0u);
@@ -411,7 +418,7 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
     const int g = lane / 4, t = lane % 4;
     const int kk[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
     uint16_t h[4], l[4];
-    for (int q = 0; q < 4; ++q) bf16_split(Bv(kk[q], g), h[q], l[q]);
+    for (int q = 0; q < 4; ++q) swe::bf16_split(Bv(kk[q], g), h[q], l[q]);
     tc[d + 0] = pack2(h[0], h[1]);
     tc[d + 1] = pack2(h[2], h[3]);
     tc[d + 2] = pack2(l[0], l[1]);
@@ -421,8 +428,8 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
   auto put8 = [&](size_t d, int lane, auto&& Bv) {
     const int g = lane / 4, t = lane % 4;
     uint16_t h0, l0, h1, l1;
-    bf16_split(Bv(2 * t, g), h0, l0);
-    bf16_split(Bv(2 * t + 1, g), h1, l1);
+    swe::bf16_split(Bv(2 * t, g), h0, l0);
+    swe::bf16_split(Bv(2 * t + 1, g), h1, l1);
     tc[d + 0] = pack2(h0, h1);
     tc[d + 1] = pack2(l0, l1);
   };
@@ -445,7 +452,7 @@ void pack_ops_n(const swe::RefElem& e, std::vector<double>& o, std::vector<uint3
         for (int ks = 0; ks < C::KSTEP; ++ks)
           put16(TL::MASS + ((((size_t)op * C::KSTEP + ks) * C::NT + nt) * 32 + lane) * 4, lane, [&](int kk, int nn) {
             const int i = 8 * nt + nn, j = 16 * ks + kk;
-            return (i < np && j < np) ? o[(op == 0 ? O::WR : O::WS) + (size_t)i * npp + j] : 0.0;
+            return (i < np && j < np) ? mass[op][(size_t)i * np + j] : 0.0;
           });
         // nodal differentiation for the strong-form pressure term, TF32 m16n8k8: lane
         // (g, t) holds column n = g, rows k = t, t + 4
