@@ -314,8 +314,9 @@ int swe_level_info(const swe_solver* solver, int32_t* L, int32_t* counts, double
  * persistent kernel that takes its work from a device queue of tickets, one ticket
  * being a tile of elements (16 of the stage kernel's phase, 32 of the TVB
  * limiter's, each phase one finest substep) of one scenario, taken by one warp. The
- * kernel's CTAs have the warps per CTA of the group's first solver
- * (swe_set_tc_warps on the tensor-core tier). Tickets are ordered phase by phase,
+ * kernel's CTAs have at most the warps per CTA of the group's first solver
+ * (swe_set_tc_warps on the tensor-core tier): several small groups share every SM, each
+ * with warps in proportion to its work. Tickets are ordered phase by phase,
  * round-robin over the scenarios, and a ticket waits (bounded in time) until every
  * tile of its scenario's earlier phases is complete, so uneven scenarios fill each
  * other's gaps. One batch step is one replay of a captured CUDA graph (per group:
@@ -391,13 +392,13 @@ int swe_set_open_faces(swe_solver* solver, const uint8_t* open);
 int swe_set_launch_config(swe_solver* solver, int32_t ctas_per_sm);
 
 /* Warps per CTA of the tensor-core stage kernel and of the persistent batch kernel
- * (FP32 tensor-core tier; default 6 at N = 1 to 3, 4 at N = 4, 7 at N = 5). Each warp
+ * (FP32 tensor-core tier; default 4 at N = 1, 2 and 4, 6 at N = 3, 7 at N = 5). Each warp
  * owns its shared-memory tiles and the CTA one copy of the operators, so more warps per
  * CTA share that copy: at N = 5 (21 KB of tiles per warp, 65 KB of operators) one CTA of
  * seven warps fits on an SM. warps in 1..8; SWE_EINVAL when that many warps' tiles do not
  * fit on an SM, SWE_EUNSUPPORTED on the other tiers. A launch with few elements uses
  * fewer warps per CTA, so that they spread over the SMs. Used by the autotuner; results do
- * not depend on it. A batch takes the warps of the first solver of each group at
+ * not depend on it. A batch takes at most the warps of the first solver of each group at
  * swe_batch_create. */
 int swe_set_tc_warps(swe_solver* solver, int32_t warps);
 

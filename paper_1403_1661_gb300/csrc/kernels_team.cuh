@@ -26,9 +26,9 @@
 //             -g eta' grad B' and the strong reference term -g h0 grad eta add up to
 //             the projection of -g h grad eta, which has no cancelling parts at all
 //             (eta = const gives zero). FP32 projects -g h' grad eta and adds the
-//             reference term as a nodal product (Team::NODAL). So only h, hu, hv and the two derivatives of
-//             eta are interpolated (five rows instead of six), two rows per momentum
-//             carry advection alone and the faces keep only the pressure jump.
+//             reference term as a nodal product (Team::NODAL). So only h, hu, hv and the
+//             two derivatives of eta are interpolated (five rows instead of six), two rows
+//             per momentum carry advection alone and the faces keep only the pressure jump.
 //   mass      hu and hv are polynomials of degree N, so their projection is one
 //             nodal operator M^-1 D^T M (all schemes: degree 2N - 1 products): two
 //             NP-long rows instead of two NCUB-long ones.
@@ -36,16 +36,16 @@
 //
 // What bounds it. FP64: the FP64 pipe (two lanes per SM and clock: a warp instruction
 // takes 16 clocks of an SM and holds its warp for 64), so what counts is the number of
-// FP64 instructions, 12.1 k per 32 elements at N = 4 (16.9 k with one thread per element
+// FP64 instructions, 12.3 k per 32 elements at N = 4 (16.9 k with one thread per element
 // and the six-row form). FP32: the shared-memory pipe (operators arrive at 128 bytes per
 // clock whether they are broadcast or not), then issue slots.
 // Measured (GB300, whole calls), one thread per element before, and now, with the overlap
 // of launches and the limiter's shorter form, which give the third case half its gain:
 //   FP64, N = 2, 512 elements, 100 single-rate steps           14.45 -> 2.55 ms
-//   FP64, N = 4, 40,185 elements, 2 macro steps of 4 levels    16.95 -> 9.48 ms (93 % of the
+//   FP64, N = 4, 40,185 elements, 2 macro steps of 4 levels    16.95 -> 9.47 ms (94 % of the
 //     FP64 pipe's issue slots in an all-active launch)
 //   FP32, N = 3, 20,480 elements, 25 limited steps              1.50 -> 1.17 ms
-//   FP32, N = 5, 75,077 elements, one R                        140.1 -> 114.6 us
+//   FP32, N = 5, 75,077 elements, one R                        139.5 -> 115.5 us
 #pragma once
 
 #include "kernels.cuh"
@@ -133,8 +133,9 @@ __device__ __forceinline__ void team_ops_ready() {
 // Lanes per element and the warp's shared tile. FP64 at N = 2 has a variant with sixteen
 // lanes (kWide; its small meshes are bound by the chain of one element: an FP64
 // instruction holds its warp for 64 cycles; team_wide in kernels_order.inc chooses),
-// everything else takes four: NB * L then equals NPP at every order and a quarter-warp's 16-byte reads of eight elements cover all banks (every element
-// stride is an odd multiple of 16 bytes).
+// everything else takes four: NB * L then equals NPP at every order and a quarter-warp's
+// 16-byte reads of eight elements cover all banks (every element stride is an odd multiple
+// of 16 bytes).
 template <typename T, int N>
 struct Team {
   using D = Dims<N>;
@@ -180,8 +181,9 @@ struct Team {
   // warps per CTA when the mesh fills the GPU: eight (two per scheduler), four where
   // their tiles would not fit on an SM (227 KB)
   // (FP32 at N = 3 and 4: six, so that two CTAs have 168 registers instead of 128, which
-  // spill: ms per macro step of 125k elements at eight and at six, cubature N = 3 0.357 and
-  // 0.336, N = 4 0.556 and 0.495; one CTA of eight 0.412 and 0.567)
+  // spill: ms per macro step of 125k elements, reference term at the points, at eight and at
+  // six, cubature N = 3 0.357 and 0.336, N = 4 0.556 and 0.495; one CTA of eight 0.412 and
+  // 0.567)
   static constexpr int MAXW = !FP64 && (D::N == 3 || D::N == 4) ? 6 : (bytes(8) <= 227 * 1024 ? 8 : 4);
   // FP32 up to N = 4 runs two CTAs per SM, the others one
   static constexpr int MINB = !FP64 && D::N <= 4 ? 2 : 1;

@@ -1888,10 +1888,15 @@ cudaError_t batch_shares(swe_batch* b, int nsm) {
     for (int q : b->groups[i].idx)
       // the instructions of an element-stage grow like Np times the points per node
       work[i] += (double)b->dofs[q] * (b->solvers[q]->N + 2) * (b->groups[i].fp64 ? 16 : 1);
-  // Only where phases are short of tickets: with more work than about seven waves of an
-  // all-active phase, full grids (one group after the other) use the GPU better
-  // (per macro step: 28 k elements 0.60 against 0.79 ms, 93 k FP32 0.35 against 0.75, but
-  // 290 k 1.67 against 1.33).
+  // Only where phases are short of tickets: with more than 54 tickets of an all-active phase
+  // per SM (131 k elements), full grids (one group after the other) use the GPU better. ms
+  // per macro step side by side | full grids, N = 3, 4 and 5, by thousands of elements:
+  //   FP32-TC, eight scenarios  95 0.62 | 0.72, 128 0.78 | 0.77, 155 0.88 | 0.82, 178 1.04 | 0.90,
+  //                             243 1.35 | 1.05
+  //   FP32-TC, six scenarios    73 0.60 | 0.75, 120 0.81 | 0.86, 164 0.98 | 1.03, 237 1.31 | 1.27
+  //   FP32, eight scenarios     95 0.67 | 0.83, 128 0.81 | 0.91, 155 0.93 | 0.98, 178 1.11 | 1.07,
+  //                             243 1.44 | 1.27
+  //   FP32, six scenarios       98 0.74 | 0.93, 138 0.92 | 1.05, 164 1.78 | 1.21, 237 2.42 | 1.52
   int64_t tickets = 0;
   for (const swe_solver* s : b->solvers) tickets += swe::batch_tiles(s->K, 0);
   if (tickets > 54 * (int64_t)nsm) return cudaSuccess;
