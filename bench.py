@@ -148,7 +148,8 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-STAGE_KERNEL_SOURCES = ("kernel_types.hpp", "kernels.cuh", "kernels_team.cuh", "kernels_tc.cuh", "kernels_order.inc")
+STAGE_KERNEL_SOURCES = ("kernel_types.hpp", "kernels.cuh", "kernels_team.cuh", "kernels_solo.cuh", "kernels_tc.cuh",
+                        "kernels_order.inc")
 
 
 def kernel_source_hash():

@@ -241,7 +241,9 @@ int swe_rhs(swe_solver* solver, void* dev_R);
  *   SWE_RHS_FUSED_SIMT  the fused kernel without tensor cores, operators in
  *                       shared memory (the solver's kernel unless SWE_FP32_TC)
  *   SWE_RHS_GLOBAL_OPS  the same, operators read from global memory through
- *                       the L1 cache (the operator placement of Section 7.4)
+ *                       the L1 cache (the operator placement of Section 7.4);
+ *                       four lanes per element also where a large FP32 set at
+ *                       N = 2 or 3 otherwise takes one thread per element
  *   SWE_RHS_SPLIT       three kernels as in Sections 7.1-7.3: traces at the
  *                       face Gauss points (Q^g) stored in device memory, the
  *                       volume term, the surface term from the stored traces

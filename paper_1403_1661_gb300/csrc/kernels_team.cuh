@@ -46,17 +46,14 @@
 //     FP64 pipe's issue slots in an all-active launch)
 //   FP32, N = 3, 20,480 elements, 25 limited steps              1.50 -> 1.17 ms
 //   FP32, N = 5, 75,077 elements, one R                        139.5 -> 115.5 us
-// Where it is the slower one: FP32 on meshes whose state and history exceed the L2 (above
-// about 150,000 elements) at N = 2 to 4, since a warp has an eighth of the elements in
-// flight over a trip to memory that one thread per element had, on half the warps. ms per
-// macro step of 4 levels, before and now, 125k | 211k | 500k elements: N = 2 0.189 and 0.184
-// | 0.287 and 0.355 | 0.559 and 0.792; N = 3 0.366 and 0.347 | 0.516 and 0.535 | 1.076 and
-// 1.178; 500k: N = 4 1.873 and 1.946, N = 5 3.699 and 3.382, collocation 0.500 and 0.751,
-// 0.806 and 0.970, 1.297 and 1.427 at N = 2, 3, 4, order-2N rules 0.529 and 0.783, 0.888 and
-// 1.031, 1.524 and 1.714. Tried: L2 prefetches a tile ahead (N = 2, 500k 0.728, but 125k 0.193
-// and N = 3, 1.28M 2.81 to 3.33), the history of all three fields at once (N = 2 0.716; the
-// tensor-core kernel, which shares the commit, 1.23 to 1.30 at N = 4), the next tile's
-// connectivity in registers (0.776), three CTAs per SM at N = 2 (0.710, 125k 0.189).
+// Where it is the slower one: FP32 on large sets, since a warp has an eighth of the elements
+// in flight over a trip to memory that one thread per element has. At N = 2 and 3 these take
+// kernels_solo.cuh. ms per macro step of 4 levels at 500k elements, one thread per element
+// before, and now: N = 4 1.873 and 1.946, order 2N 1.524 and 1.714, collocation 1.297 and
+// 1.427 (N = 5 3.699 and 3.382). Tried at N = 2, 500k elements, 0.776 to 0.792 ms: L2
+// prefetches a tile ahead (0.728, but 125k 0.185 to 0.193), the history of all three fields
+// at once (0.716; the tensor-core kernel, which shares the commit, 1.23 to 1.30 at N = 4),
+// the next tile's connectivity in registers (0.776), three CTAs per SM (0.710).
 #pragma once
 
 #include "kernels.cuh"

@@ -18,6 +18,7 @@ struct KernelCfg {
   int grid_stage = 0, grid_pos = 0, grid_tvb = 0, grid_stats = 0;
   int grid_tc = 0;                // tensor-core stage kernel (FP32 only)
   int tc_warps = 4;               // warps per CTA of the tensor-core stage and batch kernels
+  int grid_solo = 0;              // stage kernel with one thread per element (FP32, large sets)
   int grid_stage_g = 0;           // stage kernel with the operators in global memory
   int grid_split_t = 0, grid_split_v = 0, grid_split_s = 0;   // kernel-split ablation
   int occ_batch = 0;              // persistent batch kernel, SIMT body

@@ -1726,6 +1726,7 @@ int apply_launch_config(swe_solver* s) {
   };
   s->cfg = s->cfg_max;
   s->cfg.grid_stage = cap(s->cfg_max.grid_stage);
+  s->cfg.grid_solo = cap(s->cfg_max.grid_solo);
   s->cfg.grid_tc = cap(s->cfg_max.grid_tc);
   s->cfg.grid_tvb = cap(s->cfg_max.grid_tvb);
   s->cfg.grid_pos = cap(s->cfg_max.grid_pos);
